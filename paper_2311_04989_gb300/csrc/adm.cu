@@ -33,7 +33,7 @@ template <class R> __device__ __forceinline__ R cvt(double x);
 template <> __device__ __forceinline__ double cvt<double>(double x) { return x; }
 template <> __device__ __forceinline__ float cvt<float>(double x) { return d2f_rn(x); }
 template <class R> __device__ __forceinline__ R rrsqrt(R x);
-template <> __device__ __forceinline__ double rrsqrt<double>(double x) { return rsqrt(x); }
+template <> __device__ __forceinline__ double rrsqrt<double>(double x) { return rsqrt64(x); }
 template <> __device__ __forceinline__ float rrsqrt<float>(float x) { return rsqrtf(x); }
 
 // Coordinates of t, t + S, t + 2S, ... in a row-major (W, H, *) box without a division per step

@@ -324,6 +324,10 @@ int gr_mesh_create(gr_ctx* ctx, const gr_block* blocks, int32_t nblocks, int32_t
       d.N[a] = s.n[a] + 2 * s.ng;
       d.dx[a] = s.dx[a];
       d.idx[a] = 1.0 / s.dx[a];
+      d.q64[a] = 0.25 * d.idx[a];
+      d.t64[a] = 1.0 / (24.0 * s.dx[a]);
+      d.q32[a] = (float)d.q64[a];
+      d.t32[a] = (float)d.t64[a];
       for (int k = 0; k < 3; ++k) d.mdiv[a][k] = mdiv_of((unsigned)(s.n[a] + k));
       d.mdiv[a][3] = mdiv_of((unsigned)d.N[a]);
     }

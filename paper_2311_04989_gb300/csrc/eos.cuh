@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include "internal.h"
+#include "soft64.cuh"
 
 namespace grs {
 
@@ -30,6 +31,11 @@ template <> __device__ __forceinline__ float rlog1p(float x) { return log1pf(x);
 template <class R> __device__ __forceinline__ R rexpm1(R x);
 template <> __device__ __forceinline__ double rexpm1(double x) { return expm1(x); }
 template <> __device__ __forceinline__ float rexpm1(float x) { return expm1f(x); }
+
+// a / b, IEEE in both precisions
+template <class R> __device__ __forceinline__ R tdiv(R a, R b);
+template <> __device__ __forceinline__ double tdiv(double a, double b) { return div64(a, b); }
+template <> __device__ __forceinline__ float tdiv(float a, float b) { return a / b; }
 
 template <class R> __device__ __forceinline__ const TabView<R>& tab_of(const KParams& kp);
 template <> __device__ __forceinline__ const TabView<double>& tab_of<double>(const KParams& kp) { return kp.t64; }
@@ -84,7 +90,7 @@ __device__ __forceinline__ R tab_inverse_T(const TabView<R>& t, const R* __restr
   if (hint >= 0 && hint < t.n[1] - 1) {
     const R gk = tab_at(t, f, L, hint), gk1 = tab_at(t, f, L, hint + 1);
     if (gk <= y && y < gk1) {
-      const R fr = (y - gk) / (gk1 - gk);
+      const R fr = tdiv(y - gk, gk1 - gk);
       *k = hint;
       *wT = fr;
       return t.x0[1] + t.dx[1] * (R(hint) + fr);
@@ -109,7 +115,7 @@ __device__ __forceinline__ R tab_inverse_T(const TabView<R>& t, const R* __restr
     if (gm <= y) { lo = mid; glo = gm; }
     else { hi = mid; ghi = gm; }
   }
-  const R fr = (y - glo) / (ghi - glo);
+  const R fr = tdiv(y - glo, ghi - glo);
   *k = lo;
   *wT = fr;
   return t.x0[1] + t.dx[1] * (R(lo) + fr);
@@ -129,7 +135,7 @@ __device__ __forceinline__ void tab_thermo_p(const TabView<R>& t, R rho, R p, R 
   const TabLoc<R> L = tab_loc(t, rlog(rho), ye, &cl);
   int k;
   R wT;
-  const R lT = tab_inverse_T(t, t.f[0], L, rlog(p / rho), &cl, &k, &wT);
+  const R lT = tab_inverse_T(t, t.f[0], L, rlog(tdiv(p, rho)), &cl, &k, &wT);
   const R l1e = tab_T(t, t.f[1], L, k, wT);       // log(1 + eps)
   *rhoh = rho * rexp(l1e) + p;
   *cs2 = tab_T(t, t.f[2], L, k, wT);

@@ -31,6 +31,20 @@ struct DBlock {
   // compiler turns into conversions on the FP64 pipe): q = floor(e / d) = umulhi(2 e, mdiv) for 32-bit e,
   // mdiv = ceil(2^63 / d)
   unsigned long long mdiv[3][4];
+  // 1/(4 dx) and 1/(24 dx), the factors of the metric derivatives, in both precisions: formed once on the host
+  // (a division, a product and a conversion of the FP64 pipe in every cell otherwise)
+  double q64[3], t64[3];
+  float q32[3], t32[3];
+#ifdef __CUDACC__
+  template <class R> __device__ __forceinline__ R qidx(int a) const {
+    if constexpr (sizeof(R) == sizeof(float)) return q32[a];
+    else return q64[a];
+  }
+  template <class R> __device__ __forceinline__ R idx24(int a) const {
+    if constexpr (sizeof(R) == sizeof(float)) return t32[a];
+    else return t64[a];
+  }
+#endif
 };
 
 __host__ __device__ __forceinline__ unsigned long long mdiv_of(unsigned d) {

@@ -10,6 +10,7 @@
 #include "eos.cuh"
 #include "internal.h"
 #include "mlp.cuh"
+#include "soft64.cuh"
 
 namespace grs {
 
@@ -20,7 +21,7 @@ namespace grs {
 // approximate square root (PTX sqrt.approx.f32, relative error of the order of one FP32 ulp), a single
 // instruction instead of the correctly rounded sequence
 template <class R> __device__ __forceinline__ R sqrt_r(R x);
-template <> __device__ __forceinline__ double sqrt_r(double x) { return sqrt(x); }
+template <> __device__ __forceinline__ double sqrt_r(double x) { return sqrt64(x); }
 template <> __device__ __forceinline__ float sqrt_r(float x) {
   float y;
   asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -29,80 +30,20 @@ template <> __device__ __forceinline__ float sqrt_r(float x) {
 // the Lorentz factor W = sqrt(1 + u~^2), correctly rounded in both precisions: tau is formed as
 // (rho h + b^2) W^2 - rho W - ..., where the rest mass cancels, so an ulp of W costs an ulp of rho
 // against the much smaller tau
-template <class R> __device__ __forceinline__ R sqrt_w(R x) { return sqrt(x); }
+template <class R> __device__ __forceinline__ R sqrt_w(R x) { return sqrt64(x); }
 template <> __device__ __forceinline__ float sqrt_w(float x) { return sqrtf(x); }
 
 // a/b: IEEE division in FP64; the fast approximate FP32 division (2 ulp) on the mixed path
 template <class R> __device__ __forceinline__ R rdiv(R a, R b);
-template <> __device__ __forceinline__ double rdiv(double a, double b) { return a / b; }
+template <> __device__ __forceinline__ double rdiv(double a, double b) { return div64(a, b); }
 template <> __device__ __forceinline__ float rdiv(float a, float b) { return __fdividef(a, b); }
 
 template <class R> __device__ __forceinline__ R rabs(R x) { return x < R(0) ? -x : x; }
-
-// whether x is finite, from the exponent bits of its high word (integer operations only: on GB300 an
-// FP64 comparison is an instruction of the narrow FP64 pipe)
-__device__ __forceinline__ bool finite64(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
-
-// Precision conversions without the FP64 pipe (on GB300 an F2F conversion is an FP64-pipe
-// instruction, ~1/64 of the FP32 rate), in integer arithmetic on the IEEE-754 encodings.
-// FP64 -> FP32: round to nearest, ties to even, with gradual underflow (float subnormals) and
-// overflow to infinity, i.e. the IEEE conversion; NaN becomes the canonical quiet NaN of its sign.
-// FP32 -> FP64 is exact.
-__device__ __forceinline__ float d2f_rn(double x) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
-  const unsigned long long sgn = u & 0x8000000000000000ull;
-  const unsigned long long a = u ^ sgn;
-  const unsigned int s32 = (unsigned int)(sgn >> 32);
-  if (a >= 0x7FF0000000000000ull) return __uint_as_float(s32 | (a > 0x7FF0000000000000ull ? 0x7FC00000u : 0x7F800000u));
-  const int e = (int)(a >> 52);                                 // biased binary exponent of |x|
-  if (e >= 1151) return __uint_as_float(s32 | 0x7F800000u);     // |x| >= 2^128
-  if (e >= 897) {                                               // |x| >= 2^-126: a normal float
-    // drop the low 29 significand bits, rounding to nearest even; a carry out of the significand
-    // steps the exponent (and turns 2^128 into infinity); rebias the exponent by 1023 - 127
-    const unsigned long long r = a + 0x0FFFFFFFull + ((a >> 29) & 1ull);
-    return __uint_as_float(s32 | (unsigned int)((r >> 29) - (896ull << 23)));
-  }
-  if (e < 873) return __uint_as_float(s32);                     // |x| < 2^-150: rounds to zero
-  // a float subnormal: |x| = M 2^(e - 1075) with the 53-bit significand M, in units of 2^-149 that is
-  // M / 2^s with s = 926 - e in [30, 53]; round the quotient to nearest even (2^23 is the smallest normal)
-  const int s = 926 - e;
-  const unsigned long long M = (a & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
-  unsigned long long q = M >> s;
-  const unsigned long long rem = M & ((1ull << s) - 1ull), half = 1ull << (s - 1);
-  if (rem > half || (rem == half && (q & 1ull))) ++q;
-  return __uint_as_float(s32 | (unsigned int)q);
-}
-
-__device__ __forceinline__ double f2d_exact(float f) {
-  const unsigned int u = __float_as_uint(f);
-  const unsigned int sgn = u & 0x80000000u;
-  const unsigned int a = u ^ sgn;
-  if (a == 0u) return __longlong_as_double((long long)((unsigned long long)sgn << 32));
-  if (a < 0x00800000u || a >= 0x7F800000u) return (double)f;    // subnormal, inf, nan (rare)
-  const unsigned long long bits = ((unsigned long long)sgn << 32) |
-                                  ((unsigned long long)((a >> 23) + 896u) << 52) |
-                                  ((unsigned long long)(a & 0x7FFFFFu) << 29);
-  return __longlong_as_double((long long)bits);
-}
 
 template <class R> __device__ __forceinline__ double to64(R x);
 template <> __device__ __forceinline__ double to64(double x) { return x; }
 template <> __device__ __forceinline__ double to64(float x) { return f2d_exact(x); }
 
-// a - b in FP64.  For two FP32 values the difference is exact in FP64; it is formed in FP32 when it is
-// exact there too (Knuth's two-sum of a and -b has a zero error term, as for values within a factor 2
-// of each other by Sterbenz's lemma) and widened by integer operations, else by an FP64 subtraction:
-// the same value either way, mostly without the narrow FP64 pipe.
-template <class R> __device__ __forceinline__ double diff64(R a, R b);
-template <> __device__ __forceinline__ double diff64(double a, double b) { return a - b; }
-template <> __device__ __forceinline__ double diff64(float a, float b) {
-  const float s = __fsub_rn(a, b);
-  const float bp = __fsub_rn(s, a);               // the part of s that came from -b
-  const float ap = __fsub_rn(s, bp);              // the part of s that came from a
-  const float err = __fadd_rn(__fsub_rn(a, ap), __fsub_rn(__fsub_rn(0.f, b), bp));
-  if (err == 0.f && isfinite(s)) return f2d_exact(s);
-  return f2d_exact(a) - f2d_exact(b);
-}
 template <class R> __device__ __forceinline__ R rmax(R a, R b) { return a > b ? a : b; }
 template <class R> __device__ __forceinline__ R rmin(R a, R b) { return a < b ? a : b; }
 
@@ -224,7 +165,7 @@ __device__ __forceinline__ void cell_metric(const DBlock& b, const InView<R>& m,
     long long v[8];
 #pragma unroll
     for (int t = 0; t < 8; ++t) v[t] = base + vix(b, i + (t & 1), j + ((t >> 1) & 1), k + (t >> 2));
-    const R ix = R(0.25 * b.idx[0]), iy = R(0.25 * b.idx[1]), iz = R(0.25 * b.idx[2]);
+    const R ix = b.qidx<R>(0), iy = b.qidx<R>(1), iz = b.qidx<R>(2);
 #pragma unroll
     for (int c = c0; c < nc; ++c) {
       const R* a = m.M[c];
@@ -240,32 +181,40 @@ __device__ __forceinline__ void cell_metric(const DBlock& b, const InView<R>& m,
     }
   } else {
     const R w[4] = {R(-1.0 / 16), R(9.0 / 16), R(9.0 / 16), R(-1.0 / 16)};
+    auto wl = [](int k) { return k == 1 || k == 2 ? R(9.0 / 16) : R(-1.0 / 16); };   // w at a run-time index
+    // components unrolled (val and dv stay in registers), the planes of a stencil in a loop
+#pragma unroll
     for (int c = c0; c < nc; ++c) {
       const R* a = m.M[c];
       R s = 0, d0 = 0;
+#pragma unroll 1
       for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
         for (int jj = 0; jj < 4; ++jj) {
           const long long r = base + vix(b, i - 1, j - 1 + jj, k - 1 + kk);
           const R f0 = a[r], f1 = a[r + 1], f2 = a[r + 2], f3 = a[r + 3];
-          const R wjk = w[jj] * w[kk];
+          const R wjk = w[jj] * wl(kk);
           s += wjk * (w[0] * f0 + w[1] * f1 + w[2] * f2 + w[3] * f3);
           if (dv && c < 10) d0 += wjk * (R(27) * (f2 - f1) - (f3 - f0));
         }
       val[c] = s;
       if (dv && c < 10) {
-        dv[0][c] = d0 * R(1.0 / (24.0 * b.dx[0]));
+        dv[0][c] = d0 * b.idx24<R>(0);
+#pragma unroll
         for (int ax = 1; ax < 3; ++ax) {
           R acc = 0;
+#pragma unroll 1
           for (int u = 0; u < 4; ++u)
+#pragma unroll
             for (int t = 0; t < 4; ++t) {
               auto at = [&](int s4) {
                 int q[3] = {i - 1 + t, j - 1 + (ax == 2 ? u : 0), k - 1 + (ax == 1 ? u : 0)};
                 q[ax] = (ax == 1 ? j : k) - 1 + s4;
                 return a[base + vix(b, q[0], q[1], q[2])];
               };
-              acc += w[t] * w[u] * (R(27) * (at(2) - at(1)) - (at(3) - at(0)));
+              acc += w[t] * wl(u) * (R(27) * (at(2) - at(1)) - (at(3) - at(0)));
             }
-          dv[ax][c] = acc * R(1.0 / (24.0 * b.dx[ax]));
+          dv[ax][c] = acc * b.idx24<R>(ax);
         }
       }
     }
@@ -288,11 +237,15 @@ template <> __device__ __forceinline__ float xa(float a, float b) { return __fad
 template <class R> __device__ __forceinline__ R xs(R a, R b) { return a - b; }
 template <> __device__ __forceinline__ float xs(float a, float b) { return __fsub_rn(a, b); }
 
+// quotient of the PLM and PPM limiters: IEEE in both precisions
+template <class R> __device__ __forceinline__ R pdiv(R a, R b) { return div64(a, b); }
+template <> __device__ __forceinline__ float pdiv(float a, float b) { return a / b; }
+
 template <class R>
 __device__ __forceinline__ R vl_slope(R wm, R w0, R wp) {
   const R dL = xs(w0, wm), dR = xs(wp, w0);
   const R pr = xm(dL, dR);
-  return pr > R(0) ? xm(R(2), pr) / xa(dL, dR) : R(0);
+  return pr > R(0) ? pdiv(xm(R(2), pr), xa(dL, dR)) : R(0);
 }
 
 // smoothness indicators and candidate values shared by both weight forms
@@ -327,7 +280,7 @@ __device__ __forceinline__ double wenoz<double>(double v0, double v1, double v2,
   const double w0 = 0.1 * (P + t5 * (e1 * e2));
   const double w1 = 0.6 * (P + t5 * (e0 * e2));
   const double w2 = 0.3 * (P + t5 * (e0 * e1));
-  return (w0 * q[0] + w1 * q[1] + w2 * q[2]) / (w0 + w1 + w2);
+  return div64(w0 * q[0] + w1 * q[1] + w2 * q[2], w0 + w1 + w2);
 }
 
 // FP32: per-weight fast divisions on the power-of-two scaled stencil (|v| < 2), eps = 1e-30.  A
@@ -369,7 +322,7 @@ __device__ __forceinline__ double weno5<double>(double v0, double v1, double v2,
   const double e0 = (bk[0] + eps) * (bk[0] + eps), e1 = (bk[1] + eps) * (bk[1] + eps);
   const double e2 = (bk[2] + eps) * (bk[2] + eps);
   const double w0 = 0.1 * (e1 * e2), w1 = 0.6 * (e0 * e2), w2 = 0.3 * (e0 * e1);
-  return (w0 * q[0] + w1 * q[1] + w2 * q[2]) / (w0 + w1 + w2);
+  return div64(w0 * q[0] + w1 * q[1] + w2 * q[2], w0 + w1 + w2);
 }
 
 template <>
@@ -422,7 +375,7 @@ __device__ __forceinline__ void ppm_cell(R v0, R v1, R v2, R v3, R v4, R* qm, R*
       l = q;
       r = q;
     } else {
-      const R ratio = d2lim / d2;
+      const R ratio = pdiv(d2lim, d2);
       l = xa(q, xm(xs(l, q), ratio));
       r = xa(q, xm(xs(r, q), ratio));
     }
@@ -783,20 +736,32 @@ __device__ __forceinline__ void cell_sources(const CellMet<R>& M, const CellFlui
 // formed only for cells that are solved
 struct C2PMet {
   double g[6], sg, det;
-  double isg;   // 1/sqrt(gamma), formed only by the FAST form
+  double isg;   // 1/sqrt(gamma), formed only by the mixed forms
 };
 
-// FAST (the mixed stage's con2prim): sqrt(gamma) and its inverse from one reciprocal square root,
-// sg = det rsqrt(det), in place of a square root and a division
-template <bool FAST = false>
+// Forms of con2prim_cell.  PLAIN: the FP64 path and gr_con2prim, step for step the oracle's.  BRACKET: the mixed
+// stage without the FP32 pre-solve (FP32 bracket top, two-division master function).  NEWTON: the mixed stage with
+// it (Newton steps from the pre-solve's root).  BRACKET keeps its roundings whatever is done to the speed: its
+// last iterate can sit anywhere in the final bracket (1e-10 wide), set by f's rounding noise, so another
+// rounding of the inputs moves p by up to 3e-7 in cold cells; NEWTON ends at the root to rounding.
+enum { C2P_PLAIN = 0, C2P_BRACKET = 1, C2P_NEWTON = 2 };
+
+// mixed forms: sqrt(gamma) and its inverse from one reciprocal square root, sg = det rsqrt(det), in place of
+// a square root and a division
+template <int MODE>
+__device__ __forceinline__ double c2p_rsqrt(double x) {
+  if constexpr (MODE == C2P_NEWTON) return rsqrt64(x);
+  else return rsqrt(x);
+}
+template <int MODE = C2P_PLAIN>
 __device__ __forceinline__ void c2pmet_from(const double g6[6], C2PMet& M) {
   for (int c = 0; c < 6; ++c) M.g[c] = g6[c];
   M.det = det3(M.g);
-  if constexpr (FAST) {
-    M.isg = rsqrt(M.det);
+  if constexpr (MODE != C2P_PLAIN) {
+    M.isg = c2p_rsqrt<MODE>(M.det);
     M.sg = M.det * M.isg;
   } else {
-    M.sg = sqrt(M.det);
+    M.sg = sqrt64(M.det);
   }
 }
 
@@ -817,6 +782,12 @@ struct C2PVal {
   bool vcap, eclamp;
 };
 
+// v^2 above its cap, eps below 0: FP64 without the FP64 pipe
+__device__ __forceinline__ bool c2p_above(double a, double b) { return gtp64(a, b); }
+__device__ __forceinline__ bool c2p_above(float a, float b) { return a > b; }
+__device__ __forceinline__ bool c2p_neg(double a) { return neg64(a); }
+__device__ __forceinline__ bool c2p_neg(float a) { return a < 0.f; }
+
 // f(mu) = mu - 1/(nu + mu rbar^2), nu = max(nu_A, nu_B).  For the ideal gas (1 + a)(1 + eps) =
 // 1 + Gamma eps, so nu_A = (1 + Gamma eps)/W and nu_B = (1 + Gamma eps)(1 + qbar - mu rbar^2)/(1 + eps);
 // eps = W (qbar - mu rbar^2) + v^2 W^2/(1 + W) is formed over the common denominator iW (1 + iW),
@@ -827,12 +798,12 @@ __device__ __forceinline__ void c2p_master(R gam, R vmax2, const C2PInv<R>& I, R
   E.rbar2 = E.x * E.x * I.r2 + mu * E.x * (R(1) + E.x) * I.rb * I.rb;
   const R qbar = I.q - R(0.5) * I.b2 - R(0.5) * mu * mu * E.x * E.x * (I.b2 * I.r2 - I.rb * I.rb);
   E.v2 = mu * mu * E.rbar2;
-  E.vcap = E.v2 > vmax2;
+  E.vcap = c2p_above(E.v2, vmax2);
   if (E.vcap) E.v2 = vmax2;
   E.iW = sqrt_r(R(1) - E.v2);
   const R qm = qbar - mu * E.rbar2;
   E.eps = rdiv(qm * (R(1) + E.iW) + E.v2, E.iW * (R(1) + E.iW));
-  E.eclamp = E.eps < R(0);
+  E.eclamp = c2p_neg(E.eps);
   if (E.eclamp) E.eps = R(0);
   const R ge = R(1) + gam * E.eps;
   const R nuA = ge * E.iW;
@@ -854,13 +825,13 @@ __device__ __forceinline__ void c2p_master_fast(R gam, R vmax2, const C2PInv<R>&
   E.rbar2 = E.x * E.x * I.r2 + mu * E.x * (R(1) + E.x) * I.rb * I.rb;
   const R qbar = I.q - R(0.5) * I.b2 - R(0.5) * mu * mu * E.x * E.x * (I.b2 * I.r2 - I.rb * I.rb);
   E.v2 = mu * mu * E.rbar2;
-  E.vcap = E.v2 > vmax2;
+  E.vcap = c2p_above(E.v2, vmax2);
   if (E.vcap) E.v2 = vmax2;
   E.iW = sqrt_r(R(1) - E.v2);
   const R qm = qbar - mu * E.rbar2;
   const R d = E.iW * (R(1) + E.iW);
   R n = qm * (R(1) + E.iW) + E.v2;
-  E.eclamp = n < R(0);
+  E.eclamp = c2p_neg(n);
   if (E.eclamp) n = R(0);
   E.en = n;
   E.ed = d;
@@ -869,6 +840,54 @@ __device__ __forceinline__ void c2p_master_fast(R gam, R vmax2, const C2PInv<R>&
   const bool a_wins = E.iW * dn > q1 * d;
   const R P = a_wins ? E.iW : q1, Q = a_wins ? d : dn;
   E.f = mu - rdiv(Q, G * P + mu * E.rbar2 * Q);
+}
+
+// c2p_master_fast in FP64 with what does not depend on mu formed once per cell (21 FP64 instructions for 34)
+struct C2PFast {
+  double r2, b2, rb2, qh, ch;   // (r.b)^2, q - b^2/2, (b^2 r^2 - (r.b)^2)/2
+};
+__device__ __forceinline__ void c2p_master_fast64(double gam, double vmax2, const C2PFast& I, double mu, C2PVal<double>& E) {
+  E.x = div64(1.0, fma(mu, I.b2, 1.0));
+  const double y = mu * E.x, s = y * I.rb2;
+  E.rbar2 = fma(E.x, fma(E.x, I.r2, s), s);
+  const double m2 = mu * E.rbar2;
+  E.v2 = mu * m2;
+  E.vcap = gtp64(E.v2, vmax2);
+  if (E.vcap) E.v2 = vmax2;
+  E.iW = sqrt64(1.0 - E.v2);
+  const double qm = fma(-(y * y), I.ch, I.qh) - m2;
+  const double w1 = 1.0 + E.iW, d = E.iW * w1;
+  double n = fma(qm, w1, E.v2);
+  E.eclamp = neg64(n);
+  if (E.eclamp) n = 0.0;
+  E.en = n;
+  E.ed = d;
+  const double G = fma(gam, n, d), dn = d + n, q1 = 1.0 + qm;
+  const bool a_wins = !gtp64(q1 * d, E.iW * dn);
+  const double P = a_wins ? E.iW : q1, Q = a_wins ? d : dn;
+  E.f = mu - div64(Q, fma(G, P, m2 * Q));
+}
+
+// df/dmu of the ideal gas's master function in FP32 (relative error ~1e-5), for the Newton steps on the FP64
+// f: with y = mu x, x' = -b2 x^2 and y' = x^2; the capped v^2 and the clamped eps are constants
+__device__ __forceinline__ float c2p_slope32(float gam, float vmax2, const C2PInv<float>& I, float mu) {
+  const float x = __fdividef(1.f, 1.f + mu * I.b2), y = mu * x, rb2 = I.rb * I.rb, dx = -I.b2 * x * x;
+  const float R = x * x * I.r2 + y * (1.f + x) * rb2;
+  const float dR = 2.f * x * dx * I.r2 + rb2 * (x * x * (1.f + x) + y * dx);
+  const float C = I.b2 * I.r2 - rb2;
+  const float qm = I.q - 0.5f * I.b2 - 0.5f * y * y * C - mu * R;
+  const float dqm = -y * x * x * C - R - mu * dR;
+  float v2 = mu * mu * R, dv2 = mu * (2.f * R + mu * dR);
+  if (v2 > vmax2) { v2 = vmax2; dv2 = 0.f; }
+  const float w = sqrt_r(1.f - v2), dw = __fdividef(-0.5f * dv2, w), id = __fdividef(1.f, w * (1.f + w));
+  float eps = (qm * (1.f + w) + v2) * id;
+  float de = (dqm * (1.f + w) + qm * dw + dv2 - eps * dw * (1.f + 2.f * w)) * id;
+  if (eps < 0.f) { eps = 0.f; de = 0.f; }
+  const float ge = 1.f + gam * eps, dge = gam * de, ie = __fdividef(1.f, 1.f + eps);
+  const float A = ge * w, B = ge * (1.f + qm) * ie;
+  const float dn = A > B ? dge * w + ge * dw : (dge * (1.f + qm) + ge * dqm - B * de) * ie;
+  const float ig = __fdividef(1.f, (A > B ? A : B) + mu * R);
+  return 1.f + (dn + R + mu * dR) * ig * ig;
 }
 
 // The same master function with the tabulated EOS (Sec. 2.2.1, App. A): rho = D/W moved into the
@@ -882,7 +901,7 @@ __device__ __forceinline__ void c2p_master_tab(const TabView<R>& t, R vmax2, con
   E.rbar2 = E.x * E.x * I.r2 + mu * E.x * (R(1) + E.x) * I.rb * I.rb;
   const R qbar = I.q - R(0.5) * I.b2 - R(0.5) * mu * mu * E.x * E.x * (I.b2 * I.r2 - I.rb * I.rb);
   E.v2 = mu * mu * E.rbar2;
-  E.vcap = E.v2 > vmax2;
+  E.vcap = c2p_above(E.v2, vmax2);
   if (E.vcap) E.v2 = vmax2;
   E.iW = sqrt_r(R(1) - E.v2);
   const R qm = qbar - mu * E.rbar2;
@@ -959,8 +978,12 @@ __device__ __forceinline__ int illinois(Fn f, R a, R b, R fa, R fb, R tol, int m
 // ~1e-7 of their terms, so a tighter FP32 tolerance would only spend steps on noise).  Returns false when
 // the FP32 invariants are not finite or f shows no sign change; else [*lo, *hi] with f32(lo) <= 0 <=
 // f32(hi), which the FP64 solve widens slightly and verifies by the signs of the FP64 f.
+// *est (in (0, top]) and *islope (1/f' there): where the FP64 Newton steps of the mixed stage start; the
+// ideal gas's slope is c2p_slope32's, the table's the secant of the bracket.  *khint: the temperature
+// interval of the last evaluation (table).
 template <int EOS>
-__device__ __forceinline__ bool c2p_presolve32(const KParams& P, const C2PInv<double>& I64, float* lo, float* hi) {
+__device__ __forceinline__ bool c2p_presolve32(const KParams& P, const C2PInv<double>& I64, float* lo, float* hi,
+                                               float* est, float* islope, int* khint) {
   C2PInv<float> I;
   I.D = d2f_rn(I64.D); I.q = d2f_rn(I64.q); I.r2 = d2f_rn(I64.r2); I.b2 = d2f_rn(I64.b2); I.rb = d2f_rn(I64.rb);
   I.ye = d2f_rn(I64.ye);
@@ -976,36 +999,51 @@ __device__ __forceinline__ bool c2p_presolve32(const KParams& P, const C2PInv<do
   }
   C2PVal<float> E;
   int kh = -1;   // temperature interval of the last evaluation (table)
-  auto fm = [&](float mu) {
+  // one evaluation of f per pass, its use by phase: 0 f(0), 1 f(mu+), 2 f(top) where f(mu+) < 0, 3 Illinois
+  float a = 0.f, b = mup, fa = 0.f, fb = 0.f, mu = 0.f;
+  float ga = 0.f, gb = 0.f;   // f(a), f(b) as evaluated (the Illinois steps halve fa, fb)
+  int phase = 0, side = 0, k = 0;
+  for (;;) {
     if constexpr (EOS == GR_EOS_IDEAL) c2p_master_fast<float>(gam, vmax2, I, mu, E);
     else c2p_master_tab<float>(P.t32, vmax2, I, mu, E, &kh);
-    return E.f;
-  };
-  float a = 0.f, b = mup;
-  float fa = fm(a), fb = fm(b);
-  if (!(fb >= 0.f) && mup < top) { b = top; fb = fm(b); }
-  if (!(fa < 0.f) || !(fb >= 0.f)) return false;
-  int side = 0;
-  for (int k = 0; k < 12 && b - a > 1e-4f * b; ++k) {
-    float c = __fdividef(a * fb - b * fa, fb - fa);
-    if (!(c > a && c < b)) c = 0.5f * (a + b);
-    if (!(c > a && c < b)) break;
-    const float fc = fm(c);
-    if (fc == 0.f) { a = c; b = c; break; }
-    if (fc < 0.f) {
-      a = c; fa = fc;
-      if (side == -1) fb *= 0.5f;
-      side = -1;
+    const float fc = E.f;
+    if (phase == 0) { fa = ga = fc; mu = mup; phase = 1; continue; }
+    if (phase < 3) {
+      fb = gb = fc;
+      if (phase == 1 && !(fb >= 0.f) && mup < top) { b = top; mu = top; phase = 2; continue; }
+      if (!(fa < 0.f) || !(fb >= 0.f)) return false;
+      phase = 3;
     } else {
-      b = c; fb = fc;
-      if (side == +1) fa *= 0.5f;
-      side = +1;
+      if (fc == 0.f) { *islope = __fdividef(b - a, gb - ga); a = mu; b = mu; break; }
+      if (fc < 0.f) {
+        a = mu; fa = ga = fc;
+        if (side == -1) fb *= 0.5f;
+        side = -1;
+      } else {
+        b = mu; fb = gb = fc;
+        if (side == +1) fa *= 0.5f;
+        side = +1;
+      }
+      ++k;
     }
+    if (k >= 12 || !(b - a > 1e-4f * b)) break;
+    mu = __fdividef(a * fb - b * fa, fb - fa);
+    if (!(mu > a && mu < b)) mu = 0.5f * (a + b);
+    if (!(mu > a && mu < b)) break;
   }
   *lo = a;
   *hi = b;
+  *khint = kh;
+  if (b > a) *islope = __fdividef(b - a, gb - ga);
+  float c = a - ga * *islope;
+  if (!(c > a && c < b)) c = 0.5f * (a + b);
+  *est = c;
+  if constexpr (EOS == GR_EOS_IDEAL) *islope = __fdividef(1.f, c2p_slope32(gam, vmax2, I, c));
   return true;
 }
+
+// phases of con2prim_cell's bracketed solve
+enum { LO, UP, M0, M1, Z, TOP, ILL };
 
 // Invariants and root of a bracketed solve (training samples for the learned bracket)
 struct C2PRecord {
@@ -1045,7 +1083,7 @@ __device__ __forceinline__ void atm_cell(const C2PMet& M, const KParams& P, cons
   const double BBd = Bd[0] * Bl[0] + Bd[1] * Bl[1] + Bd[2] * Bl[2];
   q[0] = M.sg * P.rho_atm;
   q[1] = q[2] = q[3] = 0.0;
-  q[4] = M.sg * P.eint_atm + (BBd == 0.0 ? 0.0 : 0.5 * BBd / M.sg);
+  q[4] = M.sg * P.eint_atm + (BBd == 0.0 ? 0.0 : div64(0.5 * BBd, M.sg));
   if constexpr (EOS == GR_EOS_TABLE) {
     w[5] = P.Ye_atm;
     w[6] = P.T_atm;
@@ -1053,32 +1091,40 @@ __device__ __forceinline__ void atm_cell(const C2PMet& M, const KParams& P, cons
   }
 }
 
-// Full con2prim of one cell.  q: densitised conserved (in/out; q[5] = D Y_e with a table), Bd:
-// densitised cell field, w: primitives out (w[5], w[6] = Y_e, T with a table).
+// Full con2prim of one cell: densitised conserved variables q (q[5] = D Y_e with a table) and cell field Bd
+// -> primitives w (w[5], w[6] = Y_e, T with a table).
 // guess: GR_GUESS_NONE (bracket (0, mu+]), GR_GUESS_FP32 (c2p_presolve32's FP32 bracket widened by 4e-6
 // of its ends; it is used only if the FP64 master function changes sign across it, else the full bracket
 // is used and GR_ST_GUESS_REJECTED is set) or GR_GUESS_MLP (GR_GUESS_AUTO is resolved on the host).
-// FAST (the mixed stage): the upper end mu+ of the bracket from the auxiliary function in FP32 (its
+// MODE: the mixed forms take the upper end mu+ of the bracket from the auxiliary function in FP32 (its
 // tolerance is 1e-3; a bound that turns out too low is caught by the sign test and replaced by 1/h0),
 // and for the ideal gas the two-division form of the master function (c2p_master_fast).  The root is
-// still bracketed in FP64 to the same tolerance; only the bracket's upper end and the rounding of f
+// still found in FP64 to the same tolerance; only the bracket's upper end and the rounding of f
 // differ from the plain form.
-template <int EOS, bool FAST = false>
-__device__ __forceinline__ int con2prim_cell(const C2PMet& M, const KParams& P, double q[6],
-                                             const double Bd[3], double w[7], int* iters,
-                                             C2PRecord* rec = nullptr) {
+// site: the cell's inputs -- site.load(M, Bd, q) before the solve, site.again(M, Bd) once more where the
+// cell is reset or rebuilt (rare), so that the metric and the field do not occupy registers during the solve.
+// q: set only as *qset says: 0 unchanged, 1 D, tau[, D Y_e] moved by a limit, 2 every variable.
+template <int EOS, int MODE = C2P_PLAIN, class Site>
+__device__ __forceinline__ int con2prim_cell(const Site& site, const KParams& P, double q[6], double w[7], int* qset,
+                                             int* iters, C2PRecord* rec = nullptr) {
+  constexpr bool FAST = MODE != C2P_PLAIN;
   int st = 0;
   *iters = 0;
+  *qset = 0;
   if (rec) rec->solved = false;
-  bool finite = isfinite(q[0]) && isfinite(q[4]);
-  for (int i = 0; i < 3; ++i) finite = finite && isfinite(q[1 + i]) && isfinite(Bd[i]);
+  C2PMet M;
+  double Bd[3];
+  site.load(M, Bd, q);
+  const double sg = M.sg;
+  bool finite = finite64(q[0]) && finite64(q[4]);
+  for (int i = 0; i < 3; ++i) finite = finite && finite64(q[1 + i]) && finite64(Bd[i]);
   // table: Y_e = (D Y_e)/D moved into the table's range (App. A)
   double ye = 0.0;
   bool ye_clamped = false;
   if constexpr (EOS == GR_EOS_TABLE) {
-    finite = finite && isfinite(q[5]);
+    finite = finite && finite64(q[5]);
     const double ylo = P.t64.x0[2], yhi = P.t64.hi[2];
-    ye = (finite && q[0] != 0.0) ? q[5] / q[0] : ylo;
+    ye = (finite && q[0] != 0.0) ? div64(q[5], q[0]) : ylo;
     if (ye < ylo) { ye = ylo; ye_clamped = true; }
     if (ye > yhi) { ye = yhi; ye_clamped = true; }
   }
@@ -1086,11 +1132,11 @@ __device__ __forceinline__ int con2prim_cell(const C2PMet& M, const KParams& P, 
   const double rho_thr = P.rho_thr;
   bool atm = false, reprim = false;
   if (!finite) { st |= GR_ST_FAILED; atm = true; }
-  else if (q[0] < rho_thr * M.sg) { st |= GR_ST_ATM_THRESHOLD; atm = true; }   // D~ < rho_thr
+  else if (neg64(q[0]) || gtp64(rho_thr * sg, q[0])) { st |= GR_ST_ATM_THRESHOLD; atm = true; }   // D~ < rho_thr
   double isg = 0.0;
   if (!atm) {
     if constexpr (FAST) isg = M.isg;
-    else isg = 1.0 / M.sg;
+    else isg = div64(1.0, sg);
     double D = q[0] * isg, tau = q[4] * isg, S[3], Bu[3];
     for (int i = 0; i < 3; ++i) {
       S[i] = q[1 + i] * isg;
@@ -1100,7 +1146,7 @@ __device__ __forceinline__ int con2prim_cell(const C2PMet& M, const KParams& P, 
     lower3(M.g, Bu, Bl);
     const double BB = Bu[0] * Bl[0] + Bu[1] * Bl[1] + Bu[2] * Bl[2];
     bool qmod = false;
-    if (BB > P.M_max * D) { D = BB / P.M_max; st |= GR_ST_BD_LIMIT; qmod = true; }
+    if (gtp64(BB, P.M_max * D)) { D = BB / P.M_max; st |= GR_ST_BD_LIMIT; qmod = true; }
     // tau floor of a static cold fluid with the same field: D eps(rho = D, T_min) + B^2/2
     double eps_min = 0.0;
     if constexpr (EOS == GR_EOS_TABLE) {
@@ -1108,7 +1154,7 @@ __device__ __forceinline__ int con2prim_cell(const C2PMet& M, const KParams& P, 
       tab_p_eps_T<double>(P.t64, D, P.t64.x0[1], ye, &pm, &eps_min);
     }
     const double tau_min = D * eps_min + 0.5 * BB;
-    if (tau < tau_min) { tau = tau_min; st |= GR_ST_TAU_FLOOR; qmod = true; }
+    if (EOS ? tau < tau_min : neg64(tau) || gtp64(tau_min, tau)) { tau = tau_min; st |= GR_ST_TAU_FLOOR; qmod = true; }
     double gi[6];
     if constexpr (FAST) inv3_id(M.g, isg * isg, gi);   // 1/det = (1/sqrt(gamma))^2
     else inv3(M.g, M.det, gi);
@@ -1117,11 +1163,11 @@ __device__ __forceinline__ int con2prim_cell(const C2PMet& M, const KParams& P, 
     I.ye = ye;
     double iD, isD;
     if constexpr (FAST) {   // 1/sqrt(D) from one reciprocal square root, 1/D its square
-      isD = rsqrt(D);
+      isD = c2p_rsqrt<MODE>(D);
       iD = isD * isD;
     } else {
-      iD = 1.0 / D;
-      isD = sqrt(iD);
+      iD = div64(1.0, D);
+      isD = sqrt64(iD);
     }
     I.q = tau * iD;
     double rl[3], ru[3], bu[3];
@@ -1139,67 +1185,24 @@ __device__ __forceinline__ int con2prim_cell(const C2PMet& M, const KParams& P, 
     int nevals = 0;   // FP64 master-function evaluations (reported through *iters)
     int kh = -1;      // temperature interval of the last evaluation (table)
     bool fresh = false;   // E holds f's values at the root (the solve's last evaluation was there)
+    C2PFast J;
+    if constexpr (EOS == GR_EOS_IDEAL && MODE == C2P_NEWTON) {
+      J.r2 = I.r2;
+      J.b2 = I.b2;
+      J.rb2 = I.rb * I.rb;
+      J.qh = fma(-0.5, I.b2, I.q);
+      J.ch = 0.5 * fma(I.b2, I.r2, -J.rb2);
+    }
     auto fm = [&](double mu) {
-      ++nevals;
-      if constexpr (EOS == GR_EOS_IDEAL && FAST) c2p_master_fast<double>(gam, vmax2, I, mu, E);
+      if constexpr (EOS == GR_EOS_IDEAL && MODE == C2P_NEWTON) c2p_master_fast64(gam, vmax2, J, mu, E);
+      else if constexpr (EOS == GR_EOS_IDEAL && FAST) c2p_master_fast<double>(gam, vmax2, I, mu, E);
       else if constexpr (EOS == GR_EOS_IDEAL) c2p_master<double>(gam, vmax2, I, mu, E);
       else c2p_master_tab<double>(P.t64, vmax2, I, mu, E, &kh);
-      return E.f;
     };
-    double root = 0.0, hi;
-    int r = -1;
-    int it_master = 0;
-    if (P.c2p_guess == GR_GUESS_FP32) {
-      float lo32, hi32;
-      if (c2p_presolve32<EOS>(P, I, &lo32, &hi32)) {
-        // the FP32 bracket widened by 4e-6 of its ends (a few FP32 roundings of f near the root)
-        const double lo = f2d_exact(lo32) * (1.0 - 4e-6), up = fmin(f2d_exact(hi32) * (1.0 + 4e-6), top);
-        const double flo = fm(lo), fup = fm(up);
-        if (flo <= 0.0 && fup >= 0.0) r = illinois<double>(fm, lo, up, flo, fup, P.tol, P.max_iter, &root, &hi, &it_master, &fresh);
-      }
-      if (r != 0) st |= GR_ST_GUESS_REJECTED;
-    } else if (P.c2p_guess == GR_GUESS_MLP && P.mlp) {
-      // learned bracket: start at the network's prediction mu_hat of the root and step outwards
-      // geometrically (factor exp(delta 2^k), k = 0..5) in the direction the sign of f points,
-      // until f changes sign; that bracket, verified by the sign change, goes to the Illinois solve
-      float f[kMlpIn];
-      c2p_features(I.q, I.r2, I.b2, I.rb, f);
-      f[4] = EOS ? (float)log(D) : 0.f;
-      f[5] = EOS ? (float)ye : 0.f;
-      const float th = __ldg(P.mlp + kMlpTMean) + __ldg(P.mlp + kMlpTStd) * mlp_z(P.mlp, f);
-      const double dl = (double)__ldg(P.mlp + kMlpStep);
-      double m0 = fmin((double)__expf(th), top);
-      if (m0 > 0.0) {
-        double f0 = fm(m0);
-        if (f0 == 0.0) {
-          root = m0;
-          r = 0;
-          fresh = true;
-        } else {
-          const double dir = f0 < 0.0 ? 1.0 : -1.0;   // f < 0 below the root
-          double step = dl;
-          for (int k = 0; k < 6 && r != 0; ++k, step *= 2.0) {
-            const double m1 = fmin(m0 * exp(dir * step), top);
-            if (!(m1 > 0.0) || m1 == m0) break;
-            const double f1 = fm(m1);
-            if ((f1 < 0.0) != (f0 < 0.0) || f1 == 0.0) {
-              const double a = fmin(m0, m1), bnd = fmax(m0, m1);
-              const double fa = (a == m0) ? f0 : f1, fb = (a == m0) ? f1 : f0;
-              r = illinois<double>(fm, a, bnd, fa, fb, P.tol, P.max_iter, &root, &hi, &it_master, &fresh);
-              break;
-            }
-            m0 = m1;
-            f0 = f1;
-          }
-        }
-      }
-      if (r != 0) st |= GR_ST_GUESS_REJECTED;
-    }
-    if (r != 0) {
-      // bracket (0, mu+], mu+ from the auxiliary function on (0, 1/h0]
-      double mup = top;
+    // upper end mu+ of the full bracket, from the auxiliary function on (0, 1/h0]
+    auto bracket_top = [&]() {
+      double mup = top, hi, rt;
       int it_aux;
-      bool aux_done = false;
       if constexpr (FAST) {
         C2PInv<float> If;
         If.D = d2f_rn(I.D); If.q = d2f_rn(I.q); If.r2 = d2f_rn(I.r2); If.b2 = d2f_rn(I.b2); If.rb = d2f_rn(I.rb);
@@ -1213,40 +1216,195 @@ __device__ __forceinline__ int con2prim_cell(const C2PMet& M, const KParams& P, 
             if (illinois<float>(fa, 0.f, topf, -1.f, f1, 1e-3f, P.max_iter, &rootf, &hif, &it_aux) == 0)
               mup = fmin(f2d_exact(hif), top);
           }
-          aux_done = true;
+          return mup;
         }
       }
-      if (!aux_done) {
-        const double f1 = c2p_aux<double>(I, h0sq, top);
-        if (f1 > 0.0) {
-          auto fa = [&](double mu) { return c2p_aux<double>(I, h0sq, mu); };
-          if (illinois<double>(fa, 0.0, top, -1.0, f1, 1e-3, P.max_iter, &root, &hi, &it_aux) == 0) mup = hi;
-        }
+      const double f1 = c2p_aux<double>(I, h0sq, top);
+      if (f1 > 0.0) {
+        auto fa = [&](double mu) { return c2p_aux<double>(I, h0sq, mu); };
+        if (illinois<double>(fa, 0.0, top, -1.0, f1, 1e-3, P.max_iter, &rt, &hi, &it_aux) == 0) mup = hi;
       }
-      const double f0 = fm(0.0);
-      double fp = fm(mup);
-      if ((f0 < 0.0) == (fp < 0.0) && mup < top) { mup = top; fp = fm(mup); }
-      r = illinois<double>(fm, 0.0, mup, f0, fp, P.tol, P.max_iter, &root, &hi, &it_master, &fresh);
+      return mup;
+    };
+    double root = 0.0, mu = 0.0;
+    int r = -1;
+    bool pre = false;      // ... and bracketed the root in [lo32, hi32]
+    float lo32 = 0.f, hi32 = 0.f, est = 0.f, islope = 0.f;
+    if (MODE != C2P_BRACKET && P.c2p_guess == GR_GUESS_FP32) {
+      pre = c2p_presolve32<EOS>(P, I, &lo32, &hi32, &est, &islope, &kh);
     }
+    if constexpr (MODE == C2P_NEWTON) {
+      // Newton steps on the FP64 f from the FP32 estimate (error ~1e-7) with the FP32 slope (~1e-5, table
+      // ~1e-3), later with the FP64 secant: three evaluations in place of the two that verify a bracket and
+      // the Illinois steps after them.  f increases through its one root, so the step |f/f'| is the distance
+      // to it: the point is taken when that is far below the tolerance (at rounding, 1e-14, for the default:
+      // the next stage rounds the primitives to FP32, and a step that ends within 1e-11 turns some of those
+      // roundings over).  Otherwise the bracketed solve below decides.
+      if (pre && islope > 0.f && islope < 1e30f) {
+        double is = f2d_exact(islope), pm = 0.0, pf = 0.0;
+        mu = f2d_exact(est);
+        const double thr = fmax(1e-4 * P.tol, 4.5e-16);
+#pragma unroll 1
+        for (int k = 0; k < 6; ++k) {
+          fm(mu);
+          ++nevals;
+          const double fc = E.f;
+          double step = fc * is;
+          if (!gtp64(fabs(step), thr * mu) && finite64(step)) { r = 0; break; }
+          if (k > 0) {
+            is = div64(mu - pm, fc - pf);
+            step = fc * is;
+            if (k == 5 && !gtp64(fabs(step), P.tol * mu) && finite64(step)) { r = 0; break; }
+          }
+          pm = mu;
+          pf = fc;
+          mu = mu - step;
+          if (!(gtp64(mu, 0.0) && !gtp64(mu, top))) break;
+        }
+        if (r == 0) {
+          root = mu;
+          fresh = true;
+          // the proposed bracket would have shown no sign change
+          if (gtp64(f2d_exact(lo32) * (1.0 - 4e-6), mu) || gtp64(mu, f2d_exact(hi32) * (1.0 + 4e-6)))
+            st |= GR_ST_GUESS_REJECTED;
+        }
+      }
+    }
+    // The bracketed solve with one evaluation of f per pass (the master function is long: several inlined
+    // copies of it do not fit the instruction cache), its use by phase.  A proposed bracket first (LO, UP: the
+    // FP32 pre-solve's ends; M0, M1: the network's outward steps), then, where that fails, the full one (Z:
+    // f(0), TOP: f(mu+), and f(1/h0) where f(mu+) has f(0)'s sign); ILL: Illinois steps on [a, b].
+    double a = 0.0, b = 0.0, fa = 0.0, fb = 0.0, mstep = 0.0;
+    int side = 0, it = 0, phase = Z, mk = 0;
+    bool guessed = false;   // a proposed bracket is being tried
+    if (r == 0) {
+    } else if (MODE != C2P_BRACKET && P.c2p_guess == GR_GUESS_FP32) {
+      if (pre) {
+        // the FP32 bracket widened by 4e-6 of its ends (a few FP32 roundings of f near the root)
+        a = f2d_exact(lo32) * (1.0 - 4e-6);
+        b = fmin(f2d_exact(hi32) * (1.0 + 4e-6), top);
+        mu = a;
+        phase = LO;
+        guessed = true;
+      } else {
+        st |= GR_ST_GUESS_REJECTED;
+      }
+    } else if (P.c2p_guess == GR_GUESS_MLP && P.mlp) {
+      // learned bracket: start at the network's prediction mu_hat of the root and step outwards
+      // geometrically (factor exp(delta 2^k), k = 0..5) in the direction the sign of f points,
+      // until f changes sign; that bracket, verified by the sign change, goes to the Illinois solve
+      float f[kMlpIn];
+      c2p_features(I.q, I.r2, I.b2, I.rb, f);
+      f[4] = EOS ? (float)log(D) : 0.f;
+      f[5] = EOS ? (float)ye : 0.f;
+      const float th = __ldg(P.mlp + kMlpTMean) + __ldg(P.mlp + kMlpTStd) * mlp_z(P.mlp, f);
+      mstep = (double)__ldg(P.mlp + kMlpStep);
+      mu = fmin((double)__expf(th), top);
+      if (mu > 0.0) {
+        phase = M0;
+        guessed = true;
+      } else {
+        st |= GR_ST_GUESS_REJECTED;
+      }
+    }
+    if (r != 0 && !guessed) {
+      b = bracket_top();
+      mu = 0.0;
+    }
+    while (r != 0) {
+      fm(mu);
+      ++nevals;
+      const double fc = E.f;
+      bool start = false, full = false;   // begin Illinois on [a, b]; give the proposed bracket up
+      if (phase == ILL) {
+        ++it;
+        if (zero64(fc)) { root = mu; r = 0; fresh = true; break; }
+        if (neg64(fc) == neg64(fa)) {
+          a = mu; fa = fc;
+          if (side == -1) fb *= 0.5;
+          side = -1;
+        } else {
+          b = mu; fb = fc;
+          if (side == +1) fa *= 0.5;
+          side = +1;
+        }
+        if (b - a <= P.tol * mu) { root = mu; r = 0; fresh = true; break; }
+        if (it >= P.max_iter) { r = -2; full = true; }
+      } else if (phase == LO) {
+        fa = fc; mu = b; phase = UP;
+        continue;
+      } else if (phase == UP) {
+        fb = fc;
+        if (fa <= 0.0 && fb >= 0.0) start = true;
+        else full = true;
+      } else if (phase == Z) {
+        fa = fc; a = 0.0; mu = b; phase = TOP;
+        continue;
+      } else if (phase == TOP) {
+        fb = fc;
+        if (neg64(fa) == neg64(fb) && b < top) { b = top; mu = top; continue; }
+        start = true;
+      } else {   // M0: f at the prediction; M1: f one step outwards from a
+        if (phase == M0) {
+          if (zero64(fc)) { root = mu; r = 0; fresh = true; break; }
+          a = mu; fa = fc;
+          if (!neg64(fc)) mstep = -mstep;   // f < 0 below the root
+        } else if (neg64(fc) != neg64(fa) || zero64(fc)) {
+          if (mu < a) { b = a; fb = fa; a = mu; fa = fc; }
+          else { b = mu; fb = fc; }
+          start = true;
+        } else {
+          a = mu; fa = fc; mstep *= 2.0; ++mk;
+        }
+        if (!start) {
+          const double m1 = mk < 6 ? fmin(a * exp(mstep), top) : 0.0;
+          if (m1 > 0.0 && m1 != a) { mu = m1; phase = M1; continue; }
+          full = true;
+        }
+      }
+      if (start) {
+        it = 0; side = 0; phase = ILL;
+        if (zero64(fa)) { root = a; r = 0; break; }
+        if (zero64(fb)) { root = b; r = 0; break; }
+        if (neg64(fa) == neg64(fb)) { r = -1; full = true; }
+      }
+      if (full) {
+        if (!guessed) break;   // no root
+        guessed = false;
+        st |= GR_ST_GUESS_REJECTED;
+        r = -1;
+        b = bracket_top();
+        mu = 0.0;
+        phase = Z;
+        continue;
+      }
+      double c = div64(a * fb - b * fa, fb - fa);
+      if (!(c > a && c < b)) {
+        c = 0.5 * (a + b);
+        if (!(c > a && c < b)) { root = c; r = 0; break; }   // c itself was not evaluated
+      }
+      mu = c;
+    }
+    fresh = fresh && r == 0;
     *iters = nevals;
     if (r != 0) {
       st |= GR_ST_FAILED;
       atm = true;
     } else {
-      const double mu = root;
+      mu = root;
       if (rec) {
         rec->q = I.q; rec->r2 = I.r2; rec->b2 = I.b2; rec->rb = I.rb; rec->mu = mu; rec->D = D; rec->ye = ye;
         rec->solved = true;
       }
-      // E at the root: the solve's last evaluation is usually there already (the ideal-gas master
-      // function is a pure function of mu, so the values are the ones a new evaluation would give)
+      // E at the root: the solve's last evaluation is usually there already (the master function is a pure
+      // function of mu, so the values are the ones a new evaluation would give)
       if constexpr (EOS == GR_EOS_IDEAL && FAST) {
-        if (!fresh) c2p_master_fast<double>(gam, vmax2, I, mu, E);
-        E.eps = E.en / E.ed;
+        if (!fresh) fm(mu);
+        E.eps = div64(E.en, E.ed);
       } else if constexpr (EOS == GR_EOS_IDEAL) {
         if (!fresh) c2p_master<double>(gam, vmax2, I, mu, E);
       } else {
-        c2p_master_tab<double>(P.t64, vmax2, I, mu, E, &kh);
+        if (!fresh) c2p_master_tab<double>(P.t64, vmax2, I, mu, E, &kh);
       }
       double vu[3];
       for (int i = 0; i < 3; ++i) vu[i] = mu * E.x * (ru[i] + mu * I.rb * bu[i]);
@@ -1258,9 +1416,9 @@ __device__ __forceinline__ int con2prim_cell(const C2PMet& M, const KParams& P, 
       }
       if (E.eclamp || ye_clamped) st |= GR_ST_EOS_CLAMP;
       const double rho = EOS ? E.rho : D * E.iW;
-      if (rho < rho_thr) { st |= GR_ST_ATM_THRESHOLD; atm = true; }
+      if (gtp64(rho_thr, rho)) { st |= GR_ST_ATM_THRESHOLD; atm = true; }
       if (!atm) {
-        const double W = 1.0 / E.iW;
+        const double W = div64(1.0, E.iW);
         w[0] = rho;
         for (int i = 0; i < 3; ++i) w[1 + i] = W * vu[i];
         if constexpr (EOS == GR_EOS_IDEAL) {
@@ -1280,16 +1438,18 @@ __device__ __forceinline__ int con2prim_cell(const C2PMet& M, const KParams& P, 
           if (ye_clamped) qmod = true;
         }
         if (qmod) {
-          q[0] = M.sg * D; q[4] = M.sg * tau;
+          q[0] = sg * D; q[4] = sg * tau;
           if (EOS) q[5] = q[0] * ye;
+          *qset = 1;
         }
       }
     }
   }
-  if (atm) {
-    atm_cell<EOS>(M, P, Bd, q, w);
-  } else if (reprim) {
-    cons_at<EOS>(M, P, w, Bd, q);
+  if (atm || reprim) {
+    *qset = 2;
+    site.again(M, Bd);
+    if (atm) atm_cell<EOS>(M, P, Bd, q, w);
+    else cons_at<EOS>(M, P, w, Bd, q);
   }
   return st;
 }

@@ -1,0 +1,260 @@
+// soft64.cuh -- FP64 division, square roots, comparisons, conversions and some sums without the FP64 pipe.
+//
+// GB300 issues one FP64 warp instruction per ~70 cycles and scheduler (measured: 126 M of them in the
+// 7.43 ms of an FP64 k_faces, the pipe 87 % busy, the issue slots 7 %), and the FP64 division and square
+// root of the compiler are about eight to ten of them each.  Here the significands are divided as integers:
+// an FP32 reciprocal (square root) refined once to ~30 bits, two quotient digits from it, and an exact
+// remainder that decides the last bit -- some 60 integer and FP32 instructions, which the idle issue slots
+// take.  div64 and sqrt64 are correctly rounded (round to nearest even), so they return the bits of the IEEE
+// operations they stand for; rsqrt64 is within 0.65 ulp.  Operands or results that are zero, subnormal,
+// infinite or NaN take the operator itself (a zero dividend of div64 does not).
+#pragma once
+
+#include <cuda_runtime.h>
+#include <math.h>
+#include <stdint.h>
+
+namespace grs {
+
+// 1/x for x in [1, 2) and 1/sqrt(x) for x in [1, 4), at least 1/2; a relative error of 2^-22 is allowed for below
+#ifdef __CUDACC__
+__device__ __forceinline__ float rcp_apx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return fmaxf(y, 0.5f);
+}
+__device__ __forceinline__ float rsqrt_apx(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return fmaxf(y, 0.5f);
+}
+#else   // a host build (the CPU tests of the integer arithmetic) brings its own
+float rcp_apx(float x);
+float rsqrt_apx(float x);
+#endif
+
+__device__ __forceinline__ uint64_t bits64(double x) { return (uint64_t)__double_as_longlong(x); }
+__device__ __forceinline__ double from64(uint64_t u) { return __longlong_as_double((long long)u); }
+// low 64 bits of (hi:lo) >> s, 0 < s < 32
+__device__ __forceinline__ uint32_t fsr(uint32_t lo, uint32_t hi, int s) { return __funnelshift_r(lo, hi, s); }
+__device__ __forceinline__ uint64_t mulw(uint32_t a, uint32_t b) { return (uint64_t)a * b; }
+
+// a / b.  Significands A, B (53 bits), A doubled if below B, so the ratio r = A/B lies in [1, 2):
+//   R     reciprocal 2^84/B from below, short by at most 12 units of its 32 bits (one Newton step on the FP32
+//         reciprocal)
+//   q1    r 2^30 from below, short by at most 14;  rem = A 2^30 - q1 B < 2^57 exactly
+//   Q     q1 2^28 + (rem 2^28/B) = r 2^58 from below, short by at most 28
+//   M     round(r 2^52), or one more: (Q + 32 + 32) >> 6; the sign of A 2^53 - (2 M - 1) B (its low 64 bits:
+//         it is smaller than 2^55) tells which.  It is never zero: a quotient is never halfway between two
+//         53-bit numbers.
+__device__ __forceinline__ double div64(double a, double b) {
+  const uint64_t ua = bits64(a), ub = bits64(b);
+  const uint32_t ah = (uint32_t)(ua >> 32), bh = (uint32_t)(ub >> 32), bl = (uint32_t)ub;
+  const uint32_t ea = (ah >> 20) & 0x7ffu, eb = (bh >> 20) & 0x7ffu;
+  int e = (int)ea - (int)eb;
+  const bool az = (ua << 1) == 0;
+  // both normal and so the quotient, whichever its rounding: exponent e or e - 1
+  if (!(eb - 1u < 2046u && (az || (ea - 1u < 2046u && (uint32_t)(e + 1021) < 2045u)))) return a / b;
+  uint64_t A = (ua & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
+  const uint64_t B = (ub & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
+  const uint32_t Bh = (uint32_t)(B >> 32);
+  const int lt = A < B;
+  A <<= lt;
+  e -= lt;
+  const uint32_t Al = (uint32_t)A, Ah = (uint32_t)(A >> 32);
+  // FP32 reciprocal of the leading 23 bits (odd, so it is below 1), biased down by 2^-21
+  const float y = rcp_apx(__uint_as_float((fsr(bl, Bh, 29) & 0x7ffffeu) | 0x3f800001u));
+  const uint32_t Y = ((__float_as_uint(y) << 8) | 0x80000000u) - 2048u;
+  const uint32_t t = __umulhi(fsr(bl, Bh, 21), Y);
+  const uint32_t R = Y + __umulhi(Y, (0x80000000u - t) << 1) - 6u;
+  const uint32_t q1 = __umulhi(fsr(Al, Ah, 22), R);
+  const uint64_t p1 = mulw(q1, bl) + ((uint64_t)(q1 * Bh) << 32);
+  const uint64_t rem = (A << 30) - p1;
+  const uint32_t q2 = __umulhi((uint32_t)(rem >> 25), R);   // rem 2^27 / B
+  const uint64_t Q = ((uint64_t)q1 << 28) + ((uint64_t)q2 << 1) + 64u;
+  const uint64_t M = Q >> 6;
+  const uint32_t Ml = (uint32_t)M, Mh = (uint32_t)(M >> 32);
+  const uint64_t MB = mulw(Ml, bl) + ((uint64_t)(Ml * Bh + Mh * bl) << 32);
+  const int64_t d = (int64_t)((((A << 52) - MB) << 1) + B);
+  const uint64_t m = M + ((uint64_t)(uint32_t)(e + 1022) << 52) - (uint64_t)(d < 0);
+  const uint64_t sg = (ua ^ ub) & 0x8000000000000000ull;
+  return from64(sg | (az ? 0ull : m));
+}
+
+// sqrt(x).  X = significand, doubled for an odd exponent: s = sqrt(X/2^52) in [1, 2):
+//   Y     2^32/s from below, short by at most 16 units;  s1 = s 2^30 from below, short by at most 18
+//   rem = X 2^8 - s1^2 exactly;  Q = s 2^58 = s1 2^28 + rem 2^28/(2 s) from below, short by at most 56
+//   M     round(s 2^52) or one more, (Q + 60 + 32) >> 6; the sign of X 2^54 - (2 M - 1)^2 tells which (never zero, as above)
+__device__ __forceinline__ double sqrt64(double x) {
+  const uint64_t u = bits64(x);
+  const uint32_t h = (uint32_t)(u >> 32);
+  const uint32_t ex = h >> 20;
+  if (ex - 1u >= 2046u) return sqrt(x);   // zero, subnormal, negative, infinite, NaN
+  const int odd = (int)((ex & 1u) ^ 1u);  // the unbiased exponent ex - 1023 is odd
+  const uint64_t X = ((u & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << odd;
+  const uint32_t Xh = (uint32_t)(X >> 22);
+  // leading bits as an FP32 number in [1, 4), odd in the last place so that the result is below 1
+  const float f = __uint_as_float((0x3f800000u + ((uint32_t)odd << 23)) | (fsr((uint32_t)u, h, 29) & 0x7ffffeu) | 1u);
+  const uint32_t Y0 = ((__float_as_uint(rsqrt_apx(f)) << 8) | 0x80000000u) - 2048u;
+  const uint32_t er = 0x40000000u - __umulhi(Xh, __umulhi(Y0, Y0));
+  const uint32_t Y = Y0 + __umulhi(Y0, er << 1) - 8u;
+  const uint32_t s1 = __umulhi(Xh, Y);
+  const uint64_t rem = (X << 8) - mulw(s1, s1);
+  const uint32_t q2 = __umulhi((uint32_t)(rem >> 5), Y);   // rem 2^26 / (2 s1)
+  const uint64_t Q = ((uint64_t)s1 << 28) + ((uint64_t)q2 << 2) + 92u;
+  const uint64_t M = Q >> 6;
+  const uint64_t T = 2 * M - 1;
+  const uint32_t Tl = (uint32_t)T, Th = (uint32_t)(T >> 32);
+  const uint64_t TT = mulw(Tl, Tl) + ((uint64_t)(2u * Tl * Th) << 32);
+  const int64_t d = (int64_t)((X << 54) - TT);
+  return from64(M + ((uint64_t)((ex + 1021u) >> 1) << 52) - (uint64_t)(d < 0));
+}
+
+// 1/sqrt(x): Y as in sqrt64, then one Newton step in 64 bits: e = 1 - X Y^2 (2^62 units, below 2^35), Y (1 + e/2)
+__device__ __forceinline__ double rsqrt64(double x) {
+  const uint64_t u = bits64(x);
+  const uint32_t h = (uint32_t)(u >> 32);
+  const uint32_t ex = h >> 20;
+  if (ex - 1u >= 2046u) return rsqrt(x);
+  const int odd = (int)((ex & 1u) ^ 1u);
+  const uint64_t X = ((u & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << odd;
+  const uint32_t Xh = (uint32_t)(X >> 22);
+  const float f = __uint_as_float((0x3f800000u + ((uint32_t)odd << 23)) | (fsr((uint32_t)u, h, 29) & 0x7ffffeu) | 1u);
+  const uint32_t Y0 = ((__float_as_uint(rsqrt_apx(f)) << 8) | 0x80000000u) - 2048u;
+  const uint32_t er = 0x40000000u - __umulhi(Xh, __umulhi(Y0, Y0));
+  const uint32_t Y = Y0 + __umulhi(Y0, er << 1) - 8u;
+  const uint64_t e = 0x4000000000000000ull - __umul64hi(X << 10, mulw(Y, Y));
+  const uint64_t y = ((uint64_t)Y << 32) + (mulw(Y, (uint32_t)(e >> 4)) >> 27);   // 2^64/s from below
+  const uint64_t M = ((y >> 1) + 0x202ull) >> 10;                                 // nearest
+  // exponent: x = s^2 2^(2k), 1/sqrt(x) = (M 2^-53) 2^-k
+  const int k = ((int)ex - 1023 - odd) / 2;
+  return from64(M + ((uint64_t)(uint32_t)(1021 - k) << 52));
+}
+
+// whether x is finite, from the exponent bits of its high word (integer operations only: on GB300 an
+// FP64 comparison is an instruction of the narrow FP64 pipe)
+__device__ __forceinline__ bool finite64(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+
+// FP64 comparisons on the encodings (an FP64 comparison is an instruction of the narrow FP64 pipe)
+// x < 0, false for -0 and NaN
+__device__ __forceinline__ bool neg64(double x) {
+  return (unsigned long long)__double_as_longlong(x) - 0x8000000000000001ull < 0x7ff0000000000000ull;
+}
+// x == 0 (either sign)
+__device__ __forceinline__ bool zero64(double x) { return ((unsigned long long)__double_as_longlong(x) << 1) == 0ull; }
+// a > b for b >= 0; false for a NaN a
+__device__ __forceinline__ bool gtp64(double a, double b) {
+  const long long u = __double_as_longlong(a);
+  return u > (__double_as_longlong(b) & 0x7fffffffffffffffll) && u <= 0x7ff0000000000000ll;
+}
+
+// Precision conversions without the FP64 pipe (on GB300 an F2F conversion is an FP64-pipe
+// instruction, ~1/64 of the FP32 rate), in integer arithmetic on the IEEE-754 encodings.
+// FP64 -> FP32: round to nearest, ties to even, with gradual underflow (float subnormals) and
+// overflow to infinity, i.e. the IEEE conversion; NaN becomes the canonical quiet NaN of its sign.
+// FP32 -> FP64 is exact.
+__device__ __forceinline__ float d2f_rn(double x) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+  const unsigned long long sgn = u & 0x8000000000000000ull;
+  const unsigned long long a = u ^ sgn;
+  const unsigned int s32 = (unsigned int)(sgn >> 32);
+  if (a >= 0x7FF0000000000000ull) return __uint_as_float(s32 | (a > 0x7FF0000000000000ull ? 0x7FC00000u : 0x7F800000u));
+  const int e = (int)(a >> 52);                                 // biased binary exponent of |x|
+  if (e >= 1151) return __uint_as_float(s32 | 0x7F800000u);     // |x| >= 2^128
+  if (e >= 897) {                                               // |x| >= 2^-126: a normal float
+    // drop the low 29 significand bits, rounding to nearest even; a carry out of the significand
+    // steps the exponent (and turns 2^128 into infinity); rebias the exponent by 1023 - 127
+    const unsigned long long r = a + 0x0FFFFFFFull + ((a >> 29) & 1ull);
+    return __uint_as_float(s32 | (unsigned int)((r >> 29) - (896ull << 23)));
+  }
+  if (e < 873) return __uint_as_float(s32);                     // |x| < 2^-150: rounds to zero
+  // a float subnormal: |x| = M 2^(e - 1075) with the 53-bit significand M, in units of 2^-149 that is
+  // M / 2^s with s = 926 - e in [30, 53]; round the quotient to nearest even (2^23 is the smallest normal)
+  const int s = 926 - e;
+  const unsigned long long M = (a & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
+  unsigned long long q = M >> s;
+  const unsigned long long rem = M & ((1ull << s) - 1ull), half = 1ull << (s - 1);
+  if (rem > half || (rem == half && (q & 1ull))) ++q;
+  return __uint_as_float(s32 | (unsigned int)q);
+}
+
+__device__ __forceinline__ double f2d_exact(float f) {
+  const unsigned int u = __float_as_uint(f);
+  const unsigned int sgn = u & 0x80000000u;
+  unsigned int a = u ^ sgn, e = a >> 23;
+  if (e - 1u < 254u) {
+    e += 896u;                                    // rebias 127 -> 1023
+  } else if (a == 0u) {
+  } else if (e == 0u) {                           // a float subnormal: normalise the significand
+    const int sh = __clz((int)a) - 8;
+    a <<= sh;
+    e = 897u - (unsigned)sh;
+  } else {                                        // infinite, or NaN (made quiet)
+    e = 2047u;
+    if (a > 0x7F800000u) a |= 0x400000u;
+  }
+  return __longlong_as_double((long long)(((unsigned long long)(sgn | (e << 20)) << 32) |
+                                          ((unsigned long long)(a & 0x7FFFFFu) << 29)));
+}
+
+// a - b in FP64.  Two FP32 values: the rounded difference s and its error term (Knuth's two-sum) add up to
+// the exact one, and where the error's last bit is within 53 bits of s they are put together as integers: s
+// widened, plus the error in units of its last place (the same value an FP64 subtraction gives, without the
+// narrow FP64 pipe: the first k_ct of a 512-block RK3 step 148 -> 88 us, its FP64 instructions per face 23 -> 10).  Wider
+// apart, or with a subnormal or non-finite value, an FP64 subtraction.
+template <class R> __device__ __forceinline__ double diff64(R a, R b);
+template <> __device__ __forceinline__ double diff64(double a, double b) { return a - b; }
+template <> __device__ __forceinline__ double diff64(float a, float b) {
+  const float s = __fsub_rn(a, b);
+  const float bp = __fsub_rn(s, a);               // the part of s that came from -b
+  const float ap = __fsub_rn(s, bp);              // the part of s that came from a
+  const float err = __fadd_rn(__fsub_rn(a, ap), __fsub_rn(__fsub_rn(0.f, b), bp));
+  const unsigned int us = __float_as_uint(s), ue = __float_as_uint(err);
+  if (err == 0.f && ((us << 1) < 0xFF000000u)) return f2d_exact(s);
+  const unsigned int es = (us >> 23) & 0xFFu, ee = (ue >> 23) & 0xFFu;
+  const int sh = (int)ee - (int)es + 29;          // err = k 2^(es - 127 - 52), k = its significand << sh
+  if (es - 1u < 254u && ee != 0u && sh >= 0 && err == err) {
+    long long k = (long long)(((ue & 0x7FFFFFu) | 0x800000u) << sh);
+    if ((int)(us ^ ue) < 0) k = (us & 0x7FFFFFu) == 0u ? -2 * k : -k;   // below a power of two the units halve
+    return __longlong_as_double(__double_as_longlong(f2d_exact(s)) + k);
+  }
+  return f2d_exact(a) - f2d_exact(b);
+}
+
+// Mean of eight FP64 values in fixed point: their significands aligned to the largest exponent (60 bits, so
+// an addend is cut below 2^-59 of the largest: a smaller error than seven roundings of FP64), summed as
+// integers and rounded once.  ~110 integer instructions for eight of the FP64 pipe (560 cycles there).
+// A non-finite value gives NaN.
+__device__ __forceinline__ double mean8_64(const double f[8]) {
+  unsigned e = 0;
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    const unsigned h = (unsigned)__double2hiint(f[t]) & 0x7fffffffu;
+    e = e > h ? e : h;
+  }
+  e >>= 20;
+  if (e == 2047u) return __longlong_as_double(0x7ff8000000000000ll);
+  long long acc = 0;
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    const unsigned h = (unsigned)__double2hiint(f[t]), l = (unsigned)__double2loint(f[t]);
+    const unsigned et = (h >> 20) & 0x7ffu;
+    unsigned sh = e - et;
+    sh = sh < 63u ? sh : 63u;
+    if (et == 0u) sh = 63u;                                          // zero (a subnormal counts as zero)
+    const unsigned mh = ((h & 0xfffffu) << 7) | 0x8000000u | (l >> 25), ml = l << 7;
+    const long long m = (long long)((((unsigned long long)mh << 32) | ml) >> sh);
+    acc += (int)h < 0 ? -m : m;
+  }
+  const unsigned long long sg = acc < 0 ? 0x8000000000000000ull : 0ull;
+  const unsigned long long u = (unsigned long long)(acc < 0 ? -acc : acc);   // 8 x mean in units 2^(e - 1075 - 7)
+  if (u == 0ull) return 0.0;
+  const int z = __clzll((long long)u);                                       // leading bit at 63 - z
+  const int ex = (int)e + 1 - z;                                             // biased exponent of the mean
+  if (ex < 1) return 0.0;                                                    // below 2^-1022
+  const unsigned long long n = u << z;                                       // 64-bit significand
+  const unsigned long long r = (n >> 11) + ((n >> 10) & 1ull & ((n & 0x3ffull) || (n & 0x800ull) ? 1ull : 0ull));
+  return __longlong_as_double((long long)(sg | (((unsigned long long)(unsigned)(ex - 1) << 52) + r)));
+}
+
+}  // namespace grs

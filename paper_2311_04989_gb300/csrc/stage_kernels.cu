@@ -30,6 +30,7 @@
 #include "stage_common.cuh"
 #include "update_common.cuh"
 
+
 namespace grs {
 
 // ------------------------------------------------------------------------------------------------
@@ -334,13 +335,24 @@ __global__ void __launch_bounds__(kMaxTile) k_ct(const DBlock* __restrict__ bloc
 // ------------------------------------------------------------------------------------------------
 // k_update<R>: U' (sources in R, FP64 accumulation) and FP64 con2prim on interior cells
 // ------------------------------------------------------------------------------------------------
-// FP64 gamma_ij at a cell centre (con2prim's metric; FAST: c2pmet_from's form for the mixed stage)
-template <bool FAST = false>
+// FP64 gamma_ij at a cell centre (con2prim's metric in its form MODE)
+template <int MODE = C2P_PLAIN>
 __device__ __forceinline__ void cell_gamma64(const DBlock& b, const InView<double>& m, int i, int j, int k,
                                              C2PMet& M) {
   double val[10];
-  cell_metric<double>(b, m, m.order, i, j, k, 4, 10, val, nullptr);
-  c2pmet_from<FAST>(val + 4, M);
+  if (MODE == C2P_NEWTON && m.order == 2) {
+    const long long v0 = b.vert + vix(b, i, j, k);
+    const int sy = b.N[0] + 1, sz = sy * (b.N[1] + 1);
+#pragma unroll
+    for (int c = 4; c < 10; ++c) {
+      const double* a = m.M[c] + v0;
+      const double f[8] = {a[0], a[1], a[sy], a[sy + 1], a[sz], a[sz + 1], a[sz + sy], a[sz + sy + 1]};
+      val[c] = mean8_64(f);
+    }
+  } else {
+    cell_metric<double>(b, m, m.order, i, j, k, 4, 10, val, nullptr);
+  }
+  c2pmet_from<MODE>(val + 4, M);
 }
 
 // Conserved variable v of interior cell (i, j, k) after the stage from the workspace's face fluxes
@@ -461,44 +473,97 @@ __global__ void __launch_bounds__(kMaxTile, sizeof(R) == sizeof(float) ? 4 : 0) 
   }
 }
 
-// k_c2p: FP64 con2prim (Sec. 3.5, App. A) of the queued cells, packed densely into warps whatever the
-// pattern of atmosphere and matter cells: thread t of the grid takes jobs t, t + grid size, ...
-// R = float (the mixed stage): the cell's U' is formed here first (update_all on the FP32 inputs);
-// R = double: U' is read from Uo (left there by k_update or by the caller of gr_con2prim).
-// FAST: con2prim_cell's mixed-stage form (FP32 bracket search, two-division master function); every
-// mixed stage uses it, the fused sweep's k_c2p (R = double) included, so that both paths agree bitwise.
-template <int EOS, class R = double, bool FAST = (sizeof(R) == sizeof(float))>
-__global__ void __maxnreg__(168) k_c2p(const DBlock* __restrict__ blocks,
-                                                  const __grid_constant__ InView<R> in,
-                                                  const __grid_constant__ InView<double> in64,
-                                                  const __grid_constant__ StateView s,
-                                                  const __grid_constant__ Workspace ws,
-                                                  const __grid_constant__ KParams kp) {
+// The queued cells, packed densely into warps whatever the pattern of atmosphere and matter cells: thread t of
+// the grid takes jobs t, t + grid size, ...
+struct Job {
+  int i, j, k;
+  long long c;
+};
+__device__ __forceinline__ Job job_cell(const DBlock& b, int e) {
+  const unsigned q0 = udiv_m((unsigned)e, b.mdiv[0][0]), q1 = udiv_m(q0, b.mdiv[1][0]);
+  Job o;
+  o.i = e - (int)q0 * b.n[0];
+  o.j = (int)q0 - (int)q1 * b.n[1];
+  o.k = (int)q1;
+  o.c = b.cell + cix(b, o.i, o.j, o.k);
+  return o;
+}
+
+// k_jobs<EOS>: U' of the queued cells of the mixed stage (update_all on the FP32 inputs) into Uo.  A kernel of
+// its own: with con2prim in the same one, its registers and code kept the solve at 12 warps per SM and out of
+// the instruction cache (AMR-like batch, 256 blocks, 4.3 M cells: 3.40 ms together, 2.70 ms as two kernels at
+// 96 registers; at 80 2.79, at 128 2.77, at 168 3.02).  0.62 ms there, latency-bound.
+template <int EOS>
+__global__ void __maxnreg__(96) k_jobs(const DBlock* __restrict__ blocks, const __grid_constant__ InView<float> in,
+                       const __grid_constant__ StateView s, const __grid_constant__ Workspace ws,
+                       const __grid_constant__ KParams kp) {
   const int n = *ws.njobs;
   for (int jdx = blockIdx.x * blockDim.x + threadIdx.x; jdx < n; jdx += gridDim.x * blockDim.x) {
     const int2 job = ws.jobs[jdx];
     const DBlock b = blocks[job.x];
-    const int e = job.y;
-    const unsigned q0 = udiv_m((unsigned)e, b.mdiv[0][0]), q1 = udiv_m(q0, b.mdiv[1][0]);
-    const int i = e - (int)q0 * b.n[0], j = (int)q0 - (int)q1 * b.n[1], k = (int)q1;
-    const long long c = b.cell + cix(b, i, j, k);
-    constexpr int NQ = EOS ? 6 : 5;
-    double q[6], Bn[3], wn[7];
-    q[5] = 0.0;
-    if constexpr (sizeof(R) == sizeof(float)) {
-      CellMet<R> M32;
-      update_all<R, EOS>(b, in, s, ws, kp, i, j, k, c, q, M32);
-    } else {
+    const Job o = job_cell(b, job.y);
+    double q[6];
+    CellMet<float> M32;
+    update_all<float, EOS>(b, in, s, ws, kp, o.i, o.j, o.k, o.c, q, M32);
 #pragma unroll
-      for (int v = 0; v < NQ; ++v) q[v] = s.Uo[v][c];
+    for (int v = 0; v < (EOS ? 6 : 5); ++v) s.Uo[v][o.c] = q[v];
+  }
+}
+
+// Inputs of con2prim at one cell of the caller's pools (con2prim_cell's site)
+template <int EOS, int MODE>
+struct PoolSite {
+  const DBlock& b;
+  const InView<double>& m;
+  const double* const* U;
+  const double* const* B;
+  int i, j, k;
+  long long c;
+  __device__ __forceinline__ void load(C2PMet& M, double Bd[3], double q[6]) const {
+#pragma unroll
+    for (int v = 0; v < (EOS ? 6 : 5); ++v) q[v] = U[v][c];
+    cell_field(b, B, i, j, k, Bd);
+    cell_gamma64<MODE>(b, m, i, j, k, M);
+  }
+  __device__ __forceinline__ void again(C2PMet& M, double Bd[3]) const {
+    int x = i, y = j, z = k;
+    asm volatile("" : "+r"(x), "+r"(y), "+r"(z));   // read again, not kept
+    cell_field(b, B, x, y, z, Bd);
+    cell_gamma64<MODE>(b, m, x, y, z, M);
+  }
+};
+
+// k_c2p: FP64 con2prim (Sec. 3.5, App. A) of the queued cells from the U' in Uo (left there by k_jobs, k_update,
+// the fused sweep or the caller of gr_con2prim).
+// MODE: con2prim_cell's form; every path of a mixed stage uses the same, so that they agree bitwise.
+// Bound by the FP64 pipe (75-84 % busy).  On the AMR-like batch (256 blocks, FP32 pre-solve) the FP64
+// instructions per warp went from 640 to about 230 and the time with k_jobs from 5.09 to 2.5 ms: divisions and
+// roots as integers (soft64.cuh), one evaluation site per solve, Newton steps, the cell metric by fixed-point
+// means.  gr_con2prim on 64 x 32^3 cells 4.79 -> 2.84 ms (ideal gas), on 32 x 32^3 with the table 7.4 -> 4.5 ms.
+template <int EOS, int MODE>
+__global__ void __maxnreg__(MODE == C2P_NEWTON ? 96 : 128) k_c2p(const DBlock* __restrict__ blocks, const __grid_constant__ InView<double> in64,
+                                       const __grid_constant__ StateView s, const __grid_constant__ Workspace ws,
+                                       const __grid_constant__ KParams kp) {
+  const int n = *ws.njobs;
+  for (int jdx = blockIdx.x * blockDim.x + threadIdx.x; jdx < n; jdx += gridDim.x * blockDim.x) {
+    const int2 job = ws.jobs[jdx];
+    const DBlock& b = blocks[job.x];
+    const Job o = job_cell(b, job.y);
+    const PoolSite<EOS, MODE> site{b, in64, s.Uo, s.Bo, o.i, o.j, o.k, o.c};
+    double q[6], wn[7];
+    int qset, iters;
+    const int st = con2prim_cell<EOS, MODE>(site, kp, q, wn, &qset, &iters);
+    if (qset) {
+      s.Uo[0][o.c] = q[0];
+      s.Uo[4][o.c] = q[4];
+      if (EOS) s.Uo[5][o.c] = q[5];
+      if (qset == 2) {
+#pragma unroll
+        for (int v = 1; v < 4; ++v) s.Uo[v][o.c] = q[v];
+      }
     }
-    cell_field(b, s.Bo, i, j, k, Bn);
-    C2PMet M;
-    cell_gamma64<FAST>(b, in64, i, j, k, M);
-    int iters;
-    const int st = con2prim_cell<EOS, FAST>(M, kp, q, Bn, wn, &iters);
-    write_cell<EOS>(s, c, q, wn, st);
-    if (s.evals) s.evals[c] = iters;
+    write_prims<EOS>(s, o.c, wn, st);
+    if (s.evals) s.evals[o.c] = iters;
   }
 }
 
@@ -598,18 +663,14 @@ __global__ void __launch_bounds__(kTile) k_c2p_samples(const DBlock* __restrict_
   const DBlock b = blocks[w.block];
   int p[3];
   if (!decode<R_INTERIOR, 0>(w, b, p)) return;
-  C2PMet M;
-  cell_gamma64(b, m, p[0], p[1], p[2], M);
   const long long c = b.cell + cix(b, p[0], p[1], p[2]);
-  constexpr int NQ = EOS ? 6 : 5;
-  double q[6], Bd[3], wn[7];
-  for (int v = 0; v < NQ; ++v) q[v] = a.U[v][c];
-  cell_field(b, a.B, p[0], p[1], p[2], Bd);
+  const PoolSite<EOS, C2P_PLAIN> site{b, m, a.U, a.B, p[0], p[1], p[2], c};
+  double q[6], wn[7];
   KParams k = kp;
   k.c2p_guess = GR_GUESS_NONE;
-  int iters;
+  int qset, iters;
   C2PRecord rec;
-  const int st = con2prim_cell<EOS>(M, k, q, Bd, wn, &iters, &rec);
+  const int st = con2prim_cell<EOS>(site, k, q, wn, &qset, &iters, &rec);
   const bool ok = rec.solved && (st & (GR_ST_BD_LIMIT | GR_ST_TAU_FLOOR)) == 0;
   a.valid[c] = ok ? 1 : 0;
   float f[kMlpIn];
@@ -732,6 +793,20 @@ cudaError_t launch_cast_pool(const double* src, float* dst, long long n, cudaStr
   return cudaGetLastError();
 }
 
+// con2prim of the queued cells of a stage
+template <int EOS, int MODE>
+static void launch_c2p_m(const DBlock* blocks, const KLaunch& q, const InView<double>& in64, const StateView& s,
+                         const Workspace& ws, const KParams& kp, cudaStream_t st) {
+  k_c2p<EOS, MODE><<<stage_grid(k_c2p<EOS, MODE>, q, 0), q.threads, 0, st>>>(blocks, in64, s, ws, kp);
+}
+template <int EOS, bool MIXED>
+static void launch_c2p(const DBlock* blocks, const KLaunch& q, const InView<double>& in64, const StateView& s,
+                       const Workspace& ws, const KParams& kp, cudaStream_t st) {
+  if constexpr (!MIXED) launch_c2p_m<EOS, C2P_PLAIN>(blocks, q, in64, s, ws, kp, st);
+  else if (kp.c2p_guess == GR_GUESS_FP32) launch_c2p_m<EOS, C2P_NEWTON>(blocks, q, in64, s, ws, kp, st);
+  else launch_c2p_m<EOS, C2P_BRACKET>(blocks, q, in64, s, ws, kp, st);
+}
+
 // The mixed stage through the fused sweep: cell prep, k_fused (faces, EMFs, CT, update), con2prim of the
 // queued cells from their U' in Uo
 static cudaError_t stage_fused(const DBlock* blocks, int nblocks, const KLaunch kl[SK_N], const InView<float>& in,
@@ -751,8 +826,7 @@ static cudaError_t stage_fused(const DBlock* blocks, int nblocks, const KLaunch 
   if (q.nwork) {
     KLaunch qq = q;
     qq.nwork = (q.nwork + q.threads - 1) / q.threads;
-    k_c2p<GR_EOS_IDEAL, double, true><<<stage_grid(k_c2p<GR_EOS_IDEAL, double, true>, qq, 0), q.threads, 0, st>>>(
-        blocks, in64, in64, s, ws, kp);
+    launch_c2p<GR_EOS_IDEAL, true>(blocks, qq, in64, s, ws, kp, st);
   }
   if (ev) cudaEventRecord(ev[7], st);
   return cudaGetLastError();
@@ -811,7 +885,9 @@ static cudaError_t stage_impl(const DBlock* blocks, const KLaunch kl[SK_N], cons
   if (q.nwork) {
     KLaunch qq = q;
     qq.nwork = (q.nwork + q.threads - 1) / q.threads;   // q.nwork = the number of interior cells
-    k_c2p<EOS, R><<<stage_grid(k_c2p<EOS, R>, qq, 0), q.threads, 0, st>>>(blocks, in, in64, s, ws, kp);
+    constexpr bool mixed = sizeof(R) == sizeof(float);
+    if constexpr (mixed) k_jobs<EOS><<<stage_grid(k_jobs<EOS>, qq, 0), q.threads, 0, st>>>(blocks, in, s, ws, kp);
+    launch_c2p<EOS, mixed>(blocks, qq, in64, s, ws, kp, st);
   }
   if (ev) cudaEventRecord(ev[7], st);
   return cudaGetLastError();
@@ -870,10 +946,10 @@ cudaError_t launch_con2prim(const DBlock* blocks, const Work* work, int nwork, i
   const int grid2 = (ninterior + kTile - 1) / kTile;
   if (kp.eos == GR_EOS_TABLE) {
     k_con2prim_prep<GR_EOS_TABLE><<<nwork, kTile, 0, st>>>(blocks, work, in64, s, ws, kp);
-    k_c2p<GR_EOS_TABLE><<<grid2, kTile, 0, st>>>(blocks, in64, in64, s, ws, kp);
+    k_c2p<GR_EOS_TABLE, C2P_PLAIN><<<grid2, kTile, 0, st>>>(blocks, in64, s, ws, kp);
   } else {
     k_con2prim_prep<GR_EOS_IDEAL><<<nwork, kTile, 0, st>>>(blocks, work, in64, s, ws, kp);
-    k_c2p<GR_EOS_IDEAL><<<grid2, kTile, 0, st>>>(blocks, in64, in64, s, ws, kp);
+    k_c2p<GR_EOS_IDEAL, C2P_PLAIN><<<grid2, kTile, 0, st>>>(blocks, in64, s, ws, kp);
   }
   return cudaGetLastError();
 }

@@ -25,12 +25,10 @@ __device__ __forceinline__ void cell_field(const DBlock& b, const double* const*
   Bd[2] = 0.5 * (B[2][f2] + B[2][f2 + (long long)b.N[0] * b.N[1]]);
 }
 
+// primitives, their FP32 copies and the status of a cell
 template <int EOS>
-__device__ __forceinline__ void write_cell(const StateView& s, long long c, const double q[6], const double w[7],
-                                           int st) {
-  constexpr int NQ = EOS ? 6 : 5, NW = EOS ? 7 : 5, N32 = EOS ? 6 : 5;
-#pragma unroll
-  for (int v = 0; v < NQ; ++v) s.Uo[v][c] = q[v];
+__device__ __forceinline__ void write_prims(const StateView& s, long long c, const double w[7], int st) {
+  constexpr int NW = EOS ? 7 : 5, N32 = EOS ? 6 : 5;
 #pragma unroll
   for (int v = 0; v < NW; ++v) s.Wo[v][c] = w[v];
   if (s.Wo32[0]) {   // FP32 copies of the new primitives (the next stage's reconstruction input)
@@ -38,6 +36,14 @@ __device__ __forceinline__ void write_cell(const StateView& s, long long c, cons
     for (int v = 0; v < N32; ++v) s.Wo32[v][c] = d2f_rn(w[v]);
   }
   if (s.status) s.status[c] = (uint8_t)st;   // optional for gr_con2prim
+}
+
+template <int EOS>
+__device__ __forceinline__ void write_cell(const StateView& s, long long c, const double q[6], const double w[7],
+                                           int st) {
+#pragma unroll
+  for (int v = 0; v < (EOS ? 6 : 5); ++v) s.Uo[v][c] = q[v];
+  write_prims<EOS>(s, c, w, st);
 }
 
 // Conserved variable v of interior cell c after the stage from its source and the fluxes through its six
