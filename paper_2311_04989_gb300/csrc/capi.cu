@@ -400,15 +400,25 @@ int gr_mesh_create(gr_ctx* ctx, const gr_block* blocks, int32_t nblocks, int32_t
       }
   for (int kind = 0; kind < R_NREGION; ++kind) m->d_work[kind] = m->tw[t128][0][kind];
   // k_cellprep sweep tiles: the x-y cell plane of each block in tiles of TX <= 32 columns (equal
-  // shares of N0) by TY = kSweepThreads / TX rows
+  // shares of N0) by TY = kSweepThreads / TX rows, each walk along z cut into parts where the tiles are few
   std::vector<SweepWork> sw;
+  long long ntiles = 0;
+  for (const DBlock& d : m->h_blocks) {
+    const int nxt = (d.N[0] + 31) / 32, TX = (d.N[0] + nxt - 1) / nxt, TY = kSweepThreads / TX;
+    ntiles += (long long)((d.N[0] + TX - 1) / TX) * ((d.N[1] + TY - 1) / TY);
+  }
   for (int b = 0; b < nblocks; ++b) {
     const DBlock& d = m->h_blocks[b];
     const int nxt = (d.N[0] + 31) / 32;
     const int TX = (d.N[0] + nxt - 1) / nxt, TY = kSweepThreads / TX;
     if ((TX + 1) * (TY + 1) > kSweepVerts) { e = cudaErrorInvalidValue; break; }
     for (int y0 = 0; y0 < d.N[1]; y0 += TY)
-      for (int x0 = 0; x0 < d.N[0]; x0 += TX) sw.push_back(SweepWork{b, x0, y0, TX | (TY << 16)});
+      for (int x0 = 0; x0 < d.N[0]; x0 += TX) {
+        const int len = (int)std::max<long long>(1, (long long)d.N[2] * ntiles / kSweepTarget);
+        const int parts = (d.N[2] + len - 1) / len;
+        for (int k = 0; k < parts; ++k)
+          sw.push_back(SweepWork{b, x0, y0, TX | (TY << 16), d.N[2] * k / parts, d.N[2] * (k + 1) / parts});
+      }
   }
   if (e == cudaSuccess) e = dalloc(sizeof(SweepWork) * std::max<size_t>(1, sw.size()), (void**)&m->ws.sweep);
   if (e == cudaSuccess && !sw.empty())

@@ -104,13 +104,19 @@ struct Shadow {
   long long ncell, nface[3], nvert;   // pool extents in elements
 };
 
-// k_cellprep sweep (order-2 metric): a TX x TY tile of the x-y cell plane of one block, swept along z;
+// k_cellprep sweep (order-2 metric): a TX x TY tile of the x-y cell plane of one block, swept along z over the
+// cell planes z0 .. z1 - 1 (0 .. N2);
 // txy = TX | TY << 16 with TX <= 32, TX * TY <= kSweepThreads, (TX + 1)(TY + 1) <= kSweepVerts
 constexpr int kSweepThreads = 256;
 constexpr int kSweepVerts = 344;
 struct SweepWork {
-  int block, x0, y0, txy;
+  int block, x0, y0, txy, z0, z1;
 };
+// A mesh with few tiles cuts their walks into this many in all: six CTAs per SM (the mixed sweep holds four at
+// once, the FP64 one two), each paying one more vertex plane.  One 16^3 block (2 tiles): 29 -> 8.5 us mixed; one 64^3
+// block (21 tiles): 121 -> 20 us mixed; one ragged 20 x 17 x 24 block: 271 -> 17 us FP64; with more tiles than this
+// nothing is cut.
+constexpr int kSweepTarget = 6 * 152;
 
 // k_faces_tile: a tile of at most kTY interior rows [j0, j1) of one block, walked along z
 constexpr int kTY = 8;

@@ -130,8 +130,8 @@ __global__ void __launch_bounds__(kMaxTile) k_cellprep(const DBlock* __restrict_
 }
 
 // k_cellprep_sweep<R> (order-2 metric): the same outputs, bitwise, with each vertex of the metric read
-// from memory once per tile instead of by each of its eight cells.  One CTA per SweepWork tile walks the
-// block along z; the vertex planes z and z + 1 of the tile (with its +1 halo in x and y) sit in shared
+// from memory once per tile instead of by each of its eight cells.  One CTA per SweepWork walks its tile of the
+// block along z, or a part of it on a mesh of few tiles (kSweepTarget); the vertex planes z and z + 1 of the tile (with its +1 halo in x and y) sit in shared
 // memory (cp.async, two buffers), and each thread carries the 2 x 2 plane sums of its cell column from one
 // cell to the next: the cell value is 1/8 ((f0 + f1) + (f2 + f3)) + ((f4 + f5) + (f6 + f7)) in the
 // order cell_metric sums it, the first bracket being the previous cell's second.
@@ -185,21 +185,21 @@ __global__ void __launch_bounds__(kSweepThreads) k_cellprep_sweep(const DBlock* 
       S[c] = (a[0] + a[1]) + (a[VX] + a[VX + 1]);
     }
   };
-  const int N2 = b.N[2];
-  load_plane(0, 0);
-  load_plane(1, 1);
+  load_plane(w.z0, 0);
+  load_plane(w.z0 + 1, 1);
   sweep_wait1();
   __syncthreads();
   R S0[10], S1[10];
   if (act) plane_sum(0, S0);
-  for (int kc = 0; kc < N2; ++kc) {
-    __syncthreads();   // every thread is done with buffer kc & 1 (plane kc)
-    if (kc + 2 <= N2) load_plane(kc + 2, kc & 1);
+  for (int kc = w.z0; kc < w.z1; ++kc) {
+    const int buf = (kc - w.z0) & 1;
+    __syncthreads();   // every thread is done with plane kc's buffer
+    if (kc + 2 <= w.z1) load_plane(kc + 2, buf);
     else sweep_commit();   // an empty group keeps wait_group 1 meaning "plane kc + 1 has landed"
     sweep_wait1();
     __syncthreads();
     if (act) {
-      plane_sum((kc + 1) & 1, S1);
+      plane_sum(buf ^ 1, S1);
       R val[10];
 #pragma unroll
       for (int c = 0; c < 10; ++c) {
