@@ -32,6 +32,36 @@ __device__ __forceinline__ void face_recon(R (*st)[6], const KParams& kp, R* L, 
   }
 }
 
+// face_recon in FP64, with the variables in a loop and each one's stencil loaded where it is used: the
+// reconstruction's integer arithmetic is too long to be repeated per variable in the instruction cache, and 42
+// FP64 stencil values need not be held at once (loads: v -> pointer to cell f-3 of variable v; their latency hides
+// behind the FP64 pipe).
+template <int EOS, int METHOD, class Ptr>
+__device__ __forceinline__ void face_recon64(const Ptr& ptr, int stride, bool wide, const KParams& kp, double* L, double* Rr) {
+  constexpr int NV = EOS ? 8 : 7;
+  bool bad = false;
+#pragma unroll 1
+  for (int v = 0; v < NV; ++v) {
+    const double* a = ptr(v);
+    double s[6];
+#pragma unroll
+    for (int t = 0; t < 6; ++t) s[t] = (!wide && (t == 0 || t == 5)) ? 0.0 : a[t * stride];
+    double l, r;
+    recon<double, METHOD>(s, kp.weno_eps, &l, &r);
+    if (v == 0 || v == 4) bad = bad || !rpos(l) || !rpos(r);
+    L[v] = l;
+    Rr[v] = r;
+  }
+  if (bad) {   // a non-physical reconstructed state (rho <= 0 or p <= 0) drops the face to first order
+#pragma unroll 1
+    for (int v = 0; v < NV; ++v) {
+      const double* a = ptr(v);
+      L[v] = a[2 * stride];
+      Rr[v] = a[3 * stride];
+    }
+  }
+}
+
 // Flux of direction D from the reconstructed states L, Rr, the face metric met (alpha, beta^i, gamma_ij at
 // the face centre) and the densitised normal field Bn.  F[0..6]: fluxes of D, S_j, tau and the two
 // induction components; *ye_up (table): Y_e of the upwind state of the mass flux.

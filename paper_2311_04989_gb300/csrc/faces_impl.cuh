@@ -27,29 +27,36 @@ __device__ __forceinline__ void face_body(const Work& w, const DBlock& b, const 
   int q[3] = {p[0], p[1], p[2]};
   q[D] -= 3;
   const int c0 = ((q[2] + b.g) * b.N[1] + (q[1] + b.g)) * b.N[0] + (q[0] + b.g);
-  R st[NV][6];
   const bool wide = (b.g >= 3 || METHOD != GR_RECON_PLM);
   const R* bc1 = reinterpret_cast<const R*>(ws.bcc[t1]) + b.wcell;
   const R* bc2 = reinterpret_cast<const R*>(ws.bcc[t2]) + b.wcell;
-  const R* wp[6];
-#pragma unroll
-  for (int v = 0; v < 6; ++v) wp[v] = (v < 5 || EOS) ? in.W[v] + b.cell : nullptr;
-#pragma unroll
-  for (int t = 0; t < 6; ++t) {
-    if (!wide && (t == 0 || t == 5)) {
-#pragma unroll
-      for (int v = 0; v < NV; ++v) st[v][t] = R(0);
-      continue;
-    }
-    const int c = c0 + t * stride;
-#pragma unroll
-    for (int v = 0; v < 5; ++v) st[v][t] = wp[v][c];
-    st[5][t] = bc1[c];
-    st[6][t] = bc2[c];
-    if constexpr (EOS == GR_EOS_TABLE) st[7][t] = wp[5][c];
-  }
   R L[NV], Rr[NV];
-  face_recon<R, EOS, METHOD>(st, kp, L, Rr);
+  if constexpr (sizeof(R) == sizeof(double)) {
+    auto ptr = [&](int v) -> const R* {
+      return c0 + (v < 5 ? in.W[v] + b.cell : (v == 5 ? bc1 : (v == 6 ? bc2 : in.W[5] + b.cell)));
+    };
+    face_recon64<EOS, METHOD>(ptr, stride, wide, kp, L, Rr);
+  } else {
+    R st[NV][6];
+    const R* wp[6];
+#pragma unroll
+    for (int v = 0; v < 6; ++v) wp[v] = (v < 5 || EOS) ? in.W[v] + b.cell : nullptr;
+#pragma unroll
+    for (int t = 0; t < 6; ++t) {
+      if (!wide && (t == 0 || t == 5)) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) st[v][t] = R(0);
+        continue;
+      }
+      const int c = c0 + t * stride;
+#pragma unroll
+      for (int v = 0; v < 5; ++v) st[v][t] = wp[v][c];
+      st[5][t] = bc1[c];
+      st[6][t] = bc2[c];
+      if constexpr (EOS == GR_EOS_TABLE) st[7][t] = wp[5][c];
+    }
+    face_recon<R, EOS, METHOD>(st, kp, L, Rr);
+  }
   R met[10];
   face_metric<R>(b, in, in.order, D, p, met);
   const long long fi = fix(b, D, p[0], p[1], p[2]);
@@ -72,9 +79,12 @@ __device__ __forceinline__ void face_body(const Work& w, const DBlock& b, const 
 // FP32: at most 72 registers, so that 14 CTAs of 64 threads (the autotuned shape) fit on an SM: 28
 // warps instead of 24 at the ~80 the kernel would take, for 16-44 spilled bytes (measured on the two-star
 // workload: 3.60 ms at 80 registers, 3.47 ms at 72, 3.55 ms at 68); with a table, whose face physics
-// holds more, 80.  FP64: 168, about what the compiler takes for it unconstrained (166)
+// holds more, 80.  FP64: 128 (48 AMR-like
+// blocks: 4.60 ms; at 80 4.73, at 96 4.68, at 168 4.62).  The FP64 kernel is bound by the FP64 pipe: 7.44 ms with
+// every operation there, 6.28 ms with its divisions and roots as integers, 4.60 ms with the reconstruction in
+// shared differences, its plain products as integers and the variables in a loop
 template <class R, int EOS, int METHOD>
-__global__ void __maxnreg__(sizeof(R) == sizeof(float) ? (EOS == GR_EOS_TABLE ? 80 : 72) : 168) k_faces(const DBlock* __restrict__ blocks, const Work* __restrict__ work,
+__global__ void __maxnreg__(sizeof(R) == sizeof(float) ? (EOS == GR_EOS_TABLE ? 80 : 72) : 128) k_faces(const DBlock* __restrict__ blocks, const Work* __restrict__ work,
                                                     int nwork, const __grid_constant__ InView<R> in,
                                                     const __grid_constant__ Workspace ws,
                                                     const __grid_constant__ KParams kp) {

@@ -46,6 +46,13 @@ template <> __device__ __forceinline__ double to64(float x) { return f2d_exact(x
 
 template <class R> __device__ __forceinline__ R rmax(R a, R b) { return a > b ? a : b; }
 template <class R> __device__ __forceinline__ R rmin(R a, R b) { return a < b ? a : b; }
+template <> __device__ __forceinline__ double rmax(double a, double b) { return gt64(a, b) ? a : b; }
+template <> __device__ __forceinline__ double rmin(double a, double b) { return gt64(b, a) ? a : b; }
+// x > 0, x == 0
+template <class R> __device__ __forceinline__ bool rpos(R x) { return x > R(0); }
+template <> __device__ __forceinline__ bool rpos(double x) { return gtp64(x, 0.0); }
+template <class R> __device__ __forceinline__ bool rzero(R x) { return x == R(0); }
+template <> __device__ __forceinline__ bool rzero(double x) { return zero64(x); }
 
 // symmetric 3x3 packed as xx, xy, xz, yy, yz, zz
 __device__ __forceinline__ int sidx(int i, int j) {
@@ -248,7 +255,7 @@ __device__ __forceinline__ R vl_slope(R wm, R w0, R wp) {
   return pr > R(0) ? pdiv(xm(R(2), pr), xa(dL, dR)) : R(0);
 }
 
-// smoothness indicators and candidate values shared by both weight forms
+// smoothness indicators and candidate values
 template <class R>
 __device__ __forceinline__ void wenoz_parts(R v0, R v1, R v2, R v3, R v4, R q[3], R bk[3]) {
   q[0] = xm(xa(xs(xm(R(2), v0), xm(R(7), v1)), xm(R(11), v2)), R(1.0 / 6.0));
@@ -262,42 +269,6 @@ __device__ __forceinline__ void wenoz_parts(R v0, R v1, R v2, R v3, R v4, R q[3]
   bk[2] = xa(xm(xm(R(13.0 / 12.0), a2), a2), xm(xm(R(0.25), c2), c2));
 }
 
-// WENOZ value at the right edge of the middle cell of v0..v4.
-// FP64: the weights alpha_k = d_k (1 + tau5/e_k), e_k = beta_k + eps, are multiplied through by
-// e_0 e_1 e_2 so that one division normalises them (same weights, one FP64 division instead of
-// four).  FP32: per-weight fast divisions on the power-of-two scaled stencil.
-template <class R>
-__device__ __forceinline__ R wenoz(R v0, R v1, R v2, R v3, R v4, R eps);
-
-template <>
-__device__ __forceinline__ double wenoz<double>(double v0, double v1, double v2, double v3, double v4,
-                                                double eps) {
-  double q[3], bk[3];
-  wenoz_parts(v0, v1, v2, v3, v4, q, bk);
-  const double t5 = fabs(bk[0] - bk[2]);
-  const double e0 = bk[0] + eps, e1 = bk[1] + eps, e2 = bk[2] + eps;
-  const double P = e0 * e1 * e2;
-  const double w0 = 0.1 * (P + t5 * (e1 * e2));
-  const double w1 = 0.6 * (P + t5 * (e0 * e2));
-  const double w2 = 0.3 * (P + t5 * (e0 * e1));
-  return div64(w0 * q[0] + w1 * q[1] + w2 * q[2], w0 + w1 + w2);
-}
-
-// FP32: per-weight fast divisions on the power-of-two scaled stencil (|v| < 2), eps = 1e-30.  A
-// product form with one division would need a much larger eps to keep e0 e1 e2 a normal float,
-// which lets rough sub-stencils leak into faces between cells ~1e11 apart in density (star
-// surface against atmosphere).
-template <>
-__device__ __forceinline__ float wenoz<float>(float v0, float v1, float v2, float v3, float v4, float eps) {
-  float q[3], bk[3];
-  wenoz_parts(v0, v1, v2, v3, v4, q, bk);
-  const float t5 = fabsf(bk[0] - bk[2]);
-  const float w0 = 0.1f * (1.f + __fdividef(t5, bk[0] + eps));
-  const float w1 = 0.6f * (1.f + __fdividef(t5, bk[1] + eps));
-  const float w2 = 0.3f * (1.f + __fdividef(t5, bk[2] + eps));
-  return __fdividef(w0 * q[0] + w1 * q[1] + w2 * q[2], w0 + w1 + w2);
-}
-
 // FP32: the stencil is scaled by a power of two near its largest magnitude before the smoothness
 // indicators are formed, so that squares of tiny densities/pressures (atmosphere p ~ 1e-30) do not
 // underflow; the scaling is exact and is undone on the result.
@@ -308,26 +279,9 @@ __device__ __forceinline__ void pow2_pair(float m, float* sc, float* isc) {
   *isc = __uint_as_float((unsigned)(127 + e) << 23);                // 2^e
 }
 
-// WENO5 (Jiang & Shu) value at the right edge of the middle cell: weights d_k / (beta_k + eps)^2.
-// FP64: multiplied through by the product of the squares so that one division normalises them;
-// FP32: per-weight fast divisions with eps = 1e-18 on the scaled stencil (eps^2 stays a normal float).
-template <class R>
-__device__ __forceinline__ R weno5(R v0, R v1, R v2, R v3, R v4, R eps);
-
-template <>
-__device__ __forceinline__ double weno5<double>(double v0, double v1, double v2, double v3, double v4,
-                                                double eps) {
-  double q[3], bk[3];
-  wenoz_parts(v0, v1, v2, v3, v4, q, bk);
-  const double e0 = (bk[0] + eps) * (bk[0] + eps), e1 = (bk[1] + eps) * (bk[1] + eps);
-  const double e2 = (bk[2] + eps) * (bk[2] + eps);
-  const double w0 = 0.1 * (e1 * e2), w1 = 0.6 * (e0 * e2), w2 = 0.3 * (e0 * e1);
-  return div64(w0 * q[0] + w1 * q[1] + w2 * q[2], w0 + w1 + w2);
-}
-
-template <>
-__device__ __forceinline__ float weno5<float>(float v0, float v1, float v2, float v3, float v4, float eps) {
-  (void)eps;
+// WENO5 (Jiang & Shu) value at the right edge of the middle cell in FP32: weights d_k / (beta_k + eps)^2 by
+// per-weight fast divisions with eps = 1e-18 on the scaled stencil (eps^2 stays a normal float).
+__device__ __forceinline__ float weno5(float v0, float v1, float v2, float v3, float v4) {
   float q[3], bk[3];
   wenoz_parts(v0, v1, v2, v3, v4, q, bk);
   const float e = 1e-18f;
@@ -429,6 +383,52 @@ __device__ __forceinline__ void wenoz_pair(const float s[6], float eps, float* L
   *Rr = __fdividef(num.y, den.y);
 }
 
+// WENOZ and WENO5 of both face states in FP64, in the differences d_i = s_{i+1} - s_i of the stencil, which the
+// two states share: curvatures a_i = d_i - d_{i-1} (their squares too), indicators 4 beta = 13/3 a^2 + c^2 with
+// c = 3 d_1 - d_0, d_1 + d_2, d_3 - 3 d_2, and the states as the middle cell plus a weighted correction
+// (q - v_2 = (5 d_1 - 2 d_0)/6, (d_1 + 2 d_2)/6, (4 d_2 - d_3)/6).  The weights 0.1, 0.6, 0.3 are taken as 1, 6, 3 and
+// multiplied through, so that one division normalises them.  The R state takes the mirrored differences with
+// their signs turned, so a mirror-symmetric stencil gives L == R bitwise.  71 FP64 operations for 110 per variable,
+// 26 of them (products outside a fused multiply-add) as integers.
+__device__ __forceinline__ double weno_side64(double v2, double d0, double d1, double d2, double d3, double w0, double w1,
+                                              double w2) {
+  const double q0 = fma(-2.0, d0, mul64(5.0, d1)), q1 = fma(2.0, d2, d1), q2 = fma(4.0, d2, -d3);
+  const double m1 = mul64(6.0, w1), m2 = mul64(3.0, w2);
+  return v2 + div64(fma(m2, q2, fma(m1, q1, mul64(w0, q0))), mul64(6.0, (w0 + m1) + m2));
+}
+// beta + eps: the sum is beta itself for beta far above eps (2^54 eps)
+__device__ __forceinline__ double add_eps64(double b, double eps) {
+  const unsigned hb = (unsigned)__double2hiint(b), he = (unsigned)__double2hiint(eps);
+  return hb > he + (56u << 20) && hb < 0x7ff00000u ? b : b + eps;
+}
+template <int METHOD>
+__device__ __forceinline__ void weno_pair64(const double s[6], double eps, double* L, double* Rr) {
+  const double d0 = s[1] - s[0], d1 = s[2] - s[1], d2 = s[3] - s[2], d3 = s[4] - s[3], d4 = s[5] - s[4];
+  const double a1 = d1 - d0, a2 = d2 - d1, a3 = d3 - d2, a4 = d4 - d3;
+  const double k = 13.0 / 3.0, e4 = 4.0 * eps;
+  const double A1 = mul64(mul64(k, a1), a1), A2 = mul64(mul64(k, a2), a2);
+  const double A3 = mul64(mul64(k, a3), a3), A4 = mul64(mul64(k, a4), a4);
+  const double c0 = fma(3.0, d1, -d0), c1 = d1 + d2, c2 = fma(-3.0, d2, d3);   // L: sub-stencils 0, 1, 2
+  const double r0 = fma(3.0, d3, -d4), r1 = d3 + d2, r2 = fma(-3.0, d2, d1);   // R: mirrored
+  const double b0 = fma(c0, c0, A1), b1 = fma(c1, c1, A2), b2 = fma(c2, c2, A3);
+  const double g0 = fma(r0, r0, A4), g1 = fma(r1, r1, A3), g2 = fma(r2, r2, A2);
+#pragma unroll
+  for (int side = 0; side < 2; ++side) {
+    double e0 = add_eps64(side ? g0 : b0, e4), e1 = add_eps64(side ? g1 : b1, e4), e2 = add_eps64(side ? g2 : b2, e4);
+    double w0, w1, w2;
+    if constexpr (METHOD == GR_RECON_WENOZ) {
+      const double t5 = fabs(side ? g0 - g2 : b0 - b2);
+      const double p01 = mul64(e0, e1), p02 = mul64(e0, e2), p12 = mul64(e1, e2), P = mul64(p01, e2);
+      w0 = fma(t5, p12, P); w1 = fma(t5, p02, P); w2 = fma(t5, p01, P);
+    } else {
+      e0 = mul64(e0, e0); e1 = mul64(e1, e1); e2 = mul64(e2, e2);
+      w0 = mul64(e1, e2); w1 = mul64(e0, e2); w2 = mul64(e0, e1);
+    }
+    if (side == 0) *L = weno_side64(s[2], d0, d1, d2, d3, w0, w1, w2);
+    else *Rr = weno_side64(s[3], -d4, -d3, -d2, -d1, w0, w1, w2);
+  }
+}
+
 // Face states of the 6-cell stencil s[0..5] = cells f-3 .. f+2 by method (Sec. 3.4)
 template <class R, int METHOD>
 __device__ __forceinline__ void recon_plain(const R s[6], R eps, R* L, R* Rr) {
@@ -440,12 +440,13 @@ __device__ __forceinline__ void recon_plain(const R s[6], R eps, R* L, R* Rr) {
     if constexpr (sizeof(R) == sizeof(float)) {
       wenoz_pair(s, eps, L, Rr);
     } else {
-      *L = wenoz(s[0], s[1], s[2], s[3], s[4], eps);
-      *Rr = wenoz(s[5], s[4], s[3], s[2], s[1], eps);
+      weno_pair64<METHOD>(s, eps, L, Rr);
     }
+  } else if constexpr (method == GR_RECON_WENO5 && sizeof(R) == sizeof(double)) {
+    weno_pair64<METHOD>(s, eps, L, Rr);
   } else if constexpr (method == GR_RECON_WENO5) {
-    *L = weno5(s[0], s[1], s[2], s[3], s[4], eps);
-    *Rr = weno5(s[5], s[4], s[3], s[2], s[1], eps);
+    *L = weno5(s[0], s[1], s[2], s[3], s[4]);
+    *Rr = weno5(s[5], s[4], s[3], s[2], s[1]);
   } else {
     R lm, lp, rm, rp;
     ppm_cell(s[0], s[1], s[2], s[3], s[4], &lm, &lp);
@@ -564,7 +565,7 @@ __device__ __forceinline__ void face_state(int d, const R met[10], R sg, R gdd, 
   const R c2 = cs2 + ca2 - cs2 * ca2;
   const R v2 = v[0] * vl[0] + v[1] * vl[1] + v[2] * vl[2];
   R disc = (R(1) - v2) * (gdd * (R(1) - v2 * c2) - v[d] * v[d] * (R(1) - c2));
-  disc = disc > R(0) ? disc : R(0);
+  disc = rpos(disc) ? disc : R(0);
   const R cr = sqrt_r(c2) * sqrt_r(disc);
   const R iden = rdiv(R(1), R(1) - v2 * c2);
   const R vc = v[d] * (R(1) - c2);
@@ -579,7 +580,7 @@ __device__ __forceinline__ void hlle(const R UL[7], const R UR[7], const R FL[7]
   const R lp = rmax(R(0), rmax(lpL, lpR));
   const R lm = rmin(R(0), rmin(lmL, lmR));
   const R den = lp - lm;
-  if (den == R(0)) {
+  if (rzero(den)) {
 #pragma unroll
     for (int v = 0; v < 7; ++v) out[v] = R(0.5) * (FL[v] + FR[v]);
     return;

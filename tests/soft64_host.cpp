@@ -61,7 +61,8 @@ int main(int, char** v) {
     double a = draw(i & 1), b = draw(i & 1);
     if (i % 7 == 0) a = b * (double)(int)(rng() % 1000);
     if (i % 11 == 0) a *= 0.0;
-    bad += !same(div64(a, b), a / b);
+    bad += !same(div64(a, b), a / b) || !same(mul64(a, b), a * b);
+    bad += gt64(a, b) != (a > b) || gt64(a, a) || gt64(b, b);
     bad += neg64(a) != (a < 0) || zero64(a) != (a == 0) || finite64(a) != std::isfinite(a);
     if (b >= 0) bad += gtp64(a, b) != (a > b) || gtp64(b, b) != (b > b);
     double x = std::fabs(draw(i & 1));
