@@ -740,11 +740,13 @@ struct C2PMet {
   double isg;   // 1/sqrt(gamma), formed only by the mixed forms
 };
 
-// Forms of con2prim_cell.  PLAIN: the FP64 path and gr_con2prim, step for step the oracle's.  BRACKET: the mixed
-// stage without the FP32 pre-solve (FP32 bracket top, two-division master function).  NEWTON: the mixed stage with
-// it (Newton steps from the pre-solve's root).  BRACKET keeps its roundings whatever is done to the speed: its
-// last iterate can sit anywhere in the final bracket (1e-10 wide), set by f's rounding noise, so another
-// rounding of the inputs moves p by up to 3e-7 in cold cells; NEWTON ends at the root to rounding.
+// Forms of con2prim_cell.  PLAIN: the FP64 path and gr_con2prim, step for step the oracle's.  NEWTON: the mixed
+// stage (Newton steps from the FP32 pre-solve's root, whether or not its bracket was asked for).  BRACKET: the
+// mixed stage with a learned bracket, and the stages of an RK driver step without the pre-solve (FP32 bracket top,
+// two-division master function).  BRACKET keeps its roundings whatever is done to the speed: its last iterate can
+// sit anywhere in the final bracket (1e-10 wide), set by f's rounding noise, and the next stage of the step rounds
+// the primitives to FP32, so a better root turns some of those over (p by up to 3e-7 after the step); one stage
+// moves by less than 1e-10.
 enum { C2P_PLAIN = 0, C2P_BRACKET = 1, C2P_NEWTON = 2 };
 
 // mixed forms: sqrt(gamma) and its inverse from one reciprocal square root, sg = det rsqrt(det), in place of
@@ -1231,7 +1233,7 @@ __device__ __forceinline__ int con2prim_cell(const Site& site, const KParams& P,
     int r = -1;
     bool pre = false;      // ... and bracketed the root in [lo32, hi32]
     float lo32 = 0.f, hi32 = 0.f, est = 0.f, islope = 0.f;
-    if (MODE != C2P_BRACKET && P.c2p_guess == GR_GUESS_FP32) {
+    if (MODE == C2P_NEWTON || (MODE == C2P_PLAIN && P.c2p_guess == GR_GUESS_FP32)) {
       pre = c2p_presolve32<EOS>(P, I, &lo32, &hi32, &est, &islope, &kh);
     }
     if constexpr (MODE == C2P_NEWTON) {
@@ -1266,7 +1268,7 @@ __device__ __forceinline__ int con2prim_cell(const Site& site, const KParams& P,
           root = mu;
           fresh = true;
           // the proposed bracket would have shown no sign change
-          if (gtp64(f2d_exact(lo32) * (1.0 - 4e-6), mu) || gtp64(mu, f2d_exact(hi32) * (1.0 + 4e-6)))
+          if (P.c2p_guess == GR_GUESS_FP32 && (gtp64(f2d_exact(lo32) * (1.0 - 4e-6), mu) || gtp64(mu, f2d_exact(hi32) * (1.0 + 4e-6))))
             st |= GR_ST_GUESS_REJECTED;
         }
       }
