@@ -75,11 +75,17 @@ __device__ __forceinline__ void adm_gamma(const DBlock& b, const AdmCellArgs& a,
       R f[8];
 #pragma unroll
       for (int t = 0; t < 8; ++t) f[t] = cvt<R>(__ldg(a.g[c] + v[t]));
-      g[c] = R(0.125) * (((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])));
+      if constexpr (sizeof(R) == sizeof(double)) g[c] = mean8_64(f);
+      else g[c] = R(0.125) * (((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])));
     }
   } else {
     const R w[4] = {R(-1.0 / 16), R(9.0 / 16), R(9.0 / 16), R(-1.0 / 16)};
+#pragma unroll
     for (int c = 0; c < 6; ++c) {
+      if constexpr (sizeof(R) == sizeof(double)) {
+        g[c] = lagr_cell64(b, a.g[c], b.vert, i, j, k);
+        continue;
+      }
       R s = 0;
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk)

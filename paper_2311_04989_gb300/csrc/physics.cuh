@@ -161,6 +161,26 @@ __device__ __forceinline__ void face_metric(const DBlock& b, const InView<R>& m,
   }
 }
 
+// Order-4 cell-centre value of one FP64 vertex field: its four vertex planes in fixed point (lagr16_64), the
+// combination along z in FP64 (3 FP64 instructions for 80)
+__device__ __forceinline__ double lagr_cell64(const DBlock& b, const double* a, long long base, int i, int j, int k) {
+  double in = 0.0, out = 0.0;
+#pragma unroll 1
+  for (int kk = 0; kk < 4; ++kk) {
+    double f[16];
+#pragma unroll
+    for (int jj = 0; jj < 4; ++jj) {
+      const double* r = a + base + vix(b, i - 1, j - 1 + jj, k - 1 + kk);
+#pragma unroll
+      for (int t = 0; t < 4; ++t) f[4 * jj + t] = r[t];
+    }
+    const double q = lagr16_64(f);
+    if (kk == 0 || kk == 3) out += q;
+    else in += q;
+  }
+  return scale64<4>(fma(9.0, in, -out));
+}
+
 // Cell-centre value of components [c0, nc) and, if dv != nullptr, derivatives d_k of components
 // [0, 10) (alpha, beta, gamma), computed in R from the FP64 vertex pools.  The derivative along k is
 // written as vertex differences so that it vanishes exactly on a constant field.
@@ -179,6 +199,17 @@ __device__ __forceinline__ void cell_metric(const DBlock& b, const InView<R>& m,
       R f[8];
 #pragma unroll
       for (int t = 0; t < 8; ++t) f[t] = a[v[t]];
+      if constexpr (sizeof(R) == sizeof(double)) {   // in fixed point (FP64 pipe: 32 additions a component)
+        if (dv && c < 10) {
+          haar8_64(f, &val[c], &dv[0][c], &dv[1][c], &dv[2][c]);
+          dv[0][c] *= ix;
+          dv[1][c] *= iy;
+          dv[2][c] *= iz;
+        } else {
+          val[c] = mean8_64(f);
+        }
+        continue;
+      }
       val[c] = R(0.125) * (((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])));
       if (dv && c < 10) {
         dv[0][c] = (((f[1] - f[0]) + (f[3] - f[2])) + ((f[5] - f[4]) + (f[7] - f[6]))) * ix;
@@ -193,6 +224,12 @@ __device__ __forceinline__ void cell_metric(const DBlock& b, const InView<R>& m,
 #pragma unroll
     for (int c = c0; c < nc; ++c) {
       const R* a = m.M[c];
+      if constexpr (sizeof(R) == sizeof(double)) {
+        if (!dv || c >= 10) {   // no derivatives: by planes in fixed point
+          val[c] = lagr_cell64(b, a, base, i, j, k);
+          continue;
+        }
+      }
       R s = 0, d0 = 0;
 #pragma unroll 1
       for (int kk = 0; kk < 4; ++kk)
@@ -743,7 +780,7 @@ struct C2PMet {
 // Forms of con2prim_cell.  PLAIN: the FP64 path and gr_con2prim, step for step the oracle's.  NEWTON: the mixed
 // stage (Newton steps from the FP32 pre-solve's root, whether or not its bracket was asked for).  BRACKET: the
 // mixed stage with a learned bracket, and the stages of an RK driver step without the pre-solve (FP32 bracket top,
-// two-division master function).  BRACKET keeps its roundings whatever is done to the speed: its last iterate can
+// two-division master function).  BRACKET keeps its roundings (order-2 metric) whatever is done to the speed: its last iterate can
 // sit anywhere in the final bracket (1e-10 wide), set by f's rounding noise, and the next stage of the step rounds
 // the primitives to FP32, so a better root turns some of those over (p by up to 3e-7 after the step); one stage
 // moves by less than 1e-10.

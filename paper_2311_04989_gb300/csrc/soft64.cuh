@@ -154,6 +154,15 @@ __device__ __forceinline__ double mul64(double a, double b) {
   return from64(((ua ^ ub) & 0x8000000000000000ull) | (n + ((uint64_t)(uint32_t)(e + (int)top - 1) << 52)));
 }
 
+// x 2^-K, exactly for a normal result
+template <int K>
+__device__ __forceinline__ double scale64(double x) {
+  const uint64_t u = bits64(x);
+  const uint32_t e = (uint32_t)(u >> 52) & 0x7ffu;
+  if (e - (K + 1u) < 2046u - K) return from64(u - ((uint64_t)K << 52));
+  return x * (1.0 / (1 << K));
+}
+
 // whether x is finite, from the exponent bits of its high word (integer operations only: on GB300 an
 // FP64 comparison is an instruction of the narrow FP64 pipe)
 __device__ __forceinline__ bool finite64(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
@@ -252,40 +261,85 @@ template <> __device__ __forceinline__ double diff64(float a, float b) {
   return f2d_exact(a) - f2d_exact(b);
 }
 
-// Mean of eight FP64 values in fixed point: their significands aligned to the largest exponent (60 bits, so
-// an addend is cut below 2^-59 of the largest: a smaller error than seven roundings of FP64), summed as
-// integers and rounded once.  ~110 integer instructions for eight of the FP64 pipe (560 cycles there).
-// A non-finite value gives NaN.
-__device__ __forceinline__ double mean8_64(const double f[8]) {
-  unsigned e = 0;
+// ------------------------------------------------------------------------------------------------
+// Sums of FP64 values in fixed point: significands aligned to the largest exponent of the set, added as 64-bit
+// integers (exactly, but for what alignment cuts off a value many bits below the largest), and rounded once.
+// ~12 integer instructions a value and ~18 a result, against 70 cycles of a scheduler for each FP64 addition.
+// ------------------------------------------------------------------------------------------------
+// largest biased exponent of n values (2047: one is not finite)
+template <int N>
+__device__ __forceinline__ uint32_t fix_exp(const double* f) {
+  uint32_t e = 0;
 #pragma unroll
-  for (int t = 0; t < 8; ++t) {
-    const unsigned h = (unsigned)__double2hiint(f[t]) & 0x7fffffffu;
+  for (int t = 0; t < N; ++t) {
+    const uint32_t h = (uint32_t)__double2hiint(f[t]) & 0x7fffffffu;
     e = e > h ? e : h;
   }
-  e >>= 20;
-  if (e == 2047u) return __longlong_as_double(0x7ff8000000000000ll);
-  long long acc = 0;
-#pragma unroll
-  for (int t = 0; t < 8; ++t) {
-    const unsigned h = (unsigned)__double2hiint(f[t]), l = (unsigned)__double2loint(f[t]);
-    const unsigned et = (h >> 20) & 0x7ffu;
-    unsigned sh = e - et;
-    sh = sh < 63u ? sh : 63u;
-    if (et == 0u) sh = 63u;                                          // zero (a subnormal counts as zero)
-    const unsigned mh = ((h & 0xfffffu) << 7) | 0x8000000u | (l >> 25), ml = l << 7;
-    const long long m = (long long)((((unsigned long long)mh << 32) | ml) >> sh);
-    acc += (int)h < 0 ? -m : m;
-  }
-  const unsigned long long sg = acc < 0 ? 0x8000000000000000ull : 0ull;
-  const unsigned long long u = (unsigned long long)(acc < 0 ? -acc : acc);   // 8 x mean in units 2^(e - 1075 - 7)
+  return e >> 20;
+}
+// f in units of 2^(e - 1075 - UP) (a subnormal counts as zero); |result| < 2^(53 + UP)
+template <int UP>
+__device__ __forceinline__ int64_t fix_of(double f, uint32_t e) {
+  const uint32_t h = (uint32_t)__double2hiint(f), l = (uint32_t)__double2loint(f);
+  const uint32_t et = (h >> 20) & 0x7ffu;
+  uint32_t sh = e - et;
+  sh = sh < 63u && et != 0u ? sh : 63u;
+  const uint32_t mh = (((h & 0xfffffu) | 0x100000u) << UP) | (UP ? l >> ((32 - UP) & 31) : 0u);
+  const int64_t m = (int64_t)((((uint64_t)mh << 32) | (l << UP)) >> sh);
+  return (int32_t)h < 0 ? -m : m;
+}
+// acc 2^x, rounded to nearest even (a result below the normal range is zero, above it infinite)
+__device__ __forceinline__ double fix_round(int64_t acc, int x) {
+  const uint64_t sg = acc < 0 ? 0x8000000000000000ull : 0ull;
+  const uint64_t u = (uint64_t)(acc < 0 ? -acc : acc);
   if (u == 0ull) return 0.0;
-  const int z = __clzll((long long)u);                                       // leading bit at 63 - z
-  const int ex = (int)e + 1 - z;                                             // biased exponent of the mean
-  if (ex < 1) return 0.0;                                                    // below 2^-1022
-  const unsigned long long n = u << z;                                       // 64-bit significand
-  const unsigned long long r = (n >> 11) + ((n >> 10) & 1ull & ((n & 0x3ffull) || (n & 0x800ull) ? 1ull : 0ull));
-  return __longlong_as_double((long long)(sg | (((unsigned long long)(unsigned)(ex - 1) << 52) + r)));
+  const int z = __clzll((long long)u);
+  const int ex = 1086 - z + x;                                   // biased exponent of the leading bit
+  if (ex < 1) return 0.0;
+  if (ex > 2046) return from64(sg | 0x7ff0000000000000ull);
+  const uint64_t n = u << z;
+  const uint64_t r = (n >> 11) + ((n >> 10) & 1ull & (uint64_t)((n & 0x3ffull) != 0ull || (n & 0x800ull) != 0ull));
+  return from64(sg | (((uint64_t)(uint32_t)(ex - 1) << 52) + r));
+}
+__device__ __forceinline__ double nan64() { return from64(0x7ff8000000000000ull); }
+
+// mean of the eight vertices of a cell (index x + 2 y + 4 z)
+__device__ __forceinline__ double mean8_64(const double f[8]) {
+  const uint32_t e = fix_exp<8>(f);
+  if (e == 2047u) return nan64();
+  int64_t a = 0;
+#pragma unroll
+  for (int t = 0; t < 8; ++t) a += fix_of<7>(f[t], e);
+  return fix_round(a, (int)e - 1075 - 7 - 3);
+}
+// the mean, and the sums of the four differences along x, y and z (each zero on a constant field)
+__device__ __forceinline__ void haar8_64(const double f[8], double* mean, double* dx, double* dy, double* dz) {
+  const uint32_t e = fix_exp<8>(f);
+  if (e == 2047u) {
+    *mean = *dx = *dy = *dz = nan64();
+    return;
+  }
+  int64_t m[8];
+#pragma unroll
+  for (int t = 0; t < 8; ++t) m[t] = fix_of<7>(f[t], e);
+  const int64_t s0 = m[0] + m[1], s1 = m[2] + m[3], s2 = m[4] + m[5], s3 = m[6] + m[7];
+  const int x = (int)e - 1075 - 7;
+  *mean = fix_round((s0 + s1) + (s2 + s3), x - 3);
+  *dx = fix_round(((m[1] - m[0]) + (m[3] - m[2])) + ((m[5] - m[4]) + (m[7] - m[6])), x);
+  *dy = fix_round((s1 - s0) + (s3 - s2), x);
+  *dz = fix_round((s2 + s3) - (s0 + s1), x);
+}
+// the 4 x 4 Lagrange midpoint interpolant of a vertex plane, weights (-1, 9, 9, -1)/16 per axis; f[4 y + x]
+__device__ __forceinline__ double lagr16_64(const double f[16]) {
+  const uint32_t e = fix_exp<16>(f);
+  if (e == 2047u) return nan64();
+  int64_t r[4];
+#pragma unroll
+  for (int y = 0; y < 4; ++y) {   // 54 bits, times at most 20 per axis: 63
+    const int64_t b = fix_of<1>(f[4 * y + 1], e) + fix_of<1>(f[4 * y + 2], e);
+    r[y] = 9 * b - (fix_of<1>(f[4 * y], e) + fix_of<1>(f[4 * y + 3], e));
+  }
+  return fix_round(9 * (r[1] + r[2]) - (r[0] + r[3]), (int)e - 1075 - 1 - 8);
 }
 
 }  // namespace grs

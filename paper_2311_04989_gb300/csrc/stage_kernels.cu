@@ -340,14 +340,13 @@ template <int MODE = C2P_PLAIN>
 __device__ __forceinline__ void cell_gamma64(const DBlock& b, const InView<double>& m, int i, int j, int k,
                                              C2PMet& M) {
   double val[10];
-  if (MODE == C2P_NEWTON && m.order == 2) {
+  if (MODE == C2P_BRACKET && m.order == 2) {   // that form keeps its roundings (physics.cuh)
     const long long v0 = b.vert + vix(b, i, j, k);
     const int sy = b.N[0] + 1, sz = sy * (b.N[1] + 1);
 #pragma unroll
     for (int c = 4; c < 10; ++c) {
       const double* a = m.M[c] + v0;
-      const double f[8] = {a[0], a[1], a[sy], a[sy + 1], a[sz], a[sz + 1], a[sz + sy], a[sz + sy + 1]};
-      val[c] = mean8_64(f);
+      val[c] = 0.125 * (((a[0] + a[1]) + (a[sy] + a[sy + 1])) + ((a[sz] + a[sz + 1]) + (a[sz + sy] + a[sz + sy + 1])));
     }
   } else {
     cell_metric<double>(b, m, m.order, i, j, k, 4, 10, val, nullptr);

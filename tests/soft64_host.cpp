@@ -91,6 +91,27 @@ int main(int, char** v) {
     // each addend cut below 2^-59 of the largest, one rounding
     const double lim = std::ldexp(big, -58) + 0.502 * (std::nextafter(std::fabs(mean), INFINITY) - std::fabs(mean));
     bad += !(std::fabs((double)((long double)mean8_64(w) - sum / 8)) <= lim);
+    // the differences: each addend cut below 2^-59 of the largest, one rounding; the plane: 2^-53 of the largest
+    double hm, hd[3];
+    haar8_64(w, &hm, hd, hd + 1, hd + 2);
+    bad += !same(hm, mean8_64(w));
+    for (int d = 0; d < 3; ++d) {
+      long double z = 0;
+      for (int q = 0; q < 8; ++q) z += (q >> d & 1) ? (long double)w[q] : -(long double)w[q];
+      const double zd = std::fabs((double)z);
+      bad += !(std::fabs((double)((long double)hd[d] - z)) <= std::ldexp(big, -55) + 0.502 * (std::nextafter(zd, INFINITY) - zd));
+    }
+    double pl[16], pb = 0;
+    long double ps = 0;
+    const long double wt[4] = {-1 / 16.0L, 9 / 16.0L, 9 / 16.0L, -1 / 16.0L};
+    for (int q = 0; q < 16; ++q) {
+      pl[q] = w[rng() % 8] * (1 + 1e-3 * (double)(rng() % 100));
+      ps += wt[q & 3] * wt[q >> 2] * pl[q];
+      pb = std::fmax(pb, std::fabs(pl[q]));
+    }
+    const double pd = std::fabs((double)ps);
+    // sixteen cuts of 2^-53 of the largest with weights that add up to 25/16, one rounding
+    bad += !(std::fabs((double)((long double)lagr16_64(pl) - ps)) <= std::ldexp(pb, -53) * 1.5625 * 1.01 + 0.502 * (std::nextafter(pd, INFINITY) - pd));
   }
   printf("bad %ld rsqrt %.4f\n", bad, worst);
   return 0;
