@@ -81,7 +81,7 @@ __device__ __forceinline__ void face_body(const Work& w, const DBlock& b, const 
 // workload: 3.60 ms at 80 registers, 3.47 ms at 72, 3.55 ms at 68); with a table, whose face physics
 // holds more, 80.  FP64: 128 (48 AMR-like
 // blocks: 4.60 ms; at 80 4.73, at 96 4.68, at 168 4.62).  The FP64 kernel is bound by the FP64 pipe: 7.44 ms with
-// every operation there, 6.28 ms with its divisions and roots as integers, 4.60 ms with the reconstruction in
+// every operation there, 6.28 ms with its divisions and roots as integers, 4.5 ms with the reconstruction in
 // shared differences, its plain products as integers and the variables in a loop
 template <class R, int EOS, int METHOD>
 __global__ void __maxnreg__(sizeof(R) == sizeof(float) ? (EOS == GR_EOS_TABLE ? 80 : 72) : 128) k_faces(const DBlock* __restrict__ blocks, const Work* __restrict__ work,

@@ -38,6 +38,10 @@ template <class R> __device__ __forceinline__ R rdiv(R a, R b);
 template <> __device__ __forceinline__ double rdiv(double a, double b) { return div64(a, b); }
 template <> __device__ __forceinline__ float rdiv(float a, float b) { return __fdividef(a, b); }
 
+// x 2^-K
+template <int K> __device__ __forceinline__ double rscale(double x) { return scale64<K>(x); }
+template <int K> __device__ __forceinline__ float rscale(float x) { return x * (1.0f / (1 << K)); }
+
 template <class R> __device__ __forceinline__ R rabs(R x) { return x < R(0) ? -x : x; }
 
 template <class R> __device__ __forceinline__ double to64(R x);
@@ -48,7 +52,9 @@ template <class R> __device__ __forceinline__ R rmax(R a, R b) { return a > b ? 
 template <class R> __device__ __forceinline__ R rmin(R a, R b) { return a < b ? a : b; }
 template <> __device__ __forceinline__ double rmax(double a, double b) { return gt64(a, b) ? a : b; }
 template <> __device__ __forceinline__ double rmin(double a, double b) { return gt64(b, a) ? a : b; }
-// x > 0, x == 0
+// a > b, x > 0, x == 0
+template <class R> __device__ __forceinline__ bool rgt(R a, R b) { return a > b; }
+template <> __device__ __forceinline__ bool rgt(double a, double b) { return gt64(a, b); }
 template <class R> __device__ __forceinline__ bool rpos(R x) { return x > R(0); }
 template <> __device__ __forceinline__ bool rpos(double x) { return gtp64(x, 0.0); }
 template <class R> __device__ __forceinline__ bool rzero(R x) { return x == R(0); }
@@ -142,7 +148,7 @@ __device__ __forceinline__ void face_metric(const DBlock& b, const InView<R>& m,
 #pragma unroll
     for (int c = 0; c < 10; ++c) {
       const R* a = m.M[c] + base + v00;
-      out[c] = R(0.25) * ((a[0] + a[s1]) + (a[s2] + a[s1 + s2]));
+            out[c] = rscale<2>((a[0] + a[s1]) + (a[s2] + a[s1 + s2]));
     }
   } else {
     const R w[4] = {R(-1.0 / 16), R(9.0 / 16), R(9.0 / 16), R(-1.0 / 16)};
@@ -426,7 +432,8 @@ __device__ __forceinline__ void wenoz_pair(const float s[6], float eps, float* L
 // (q - v_2 = (5 d_1 - 2 d_0)/6, (d_1 + 2 d_2)/6, (4 d_2 - d_3)/6).  The weights 0.1, 0.6, 0.3 are taken as 1, 6, 3 and
 // multiplied through, so that one division normalises them.  The R state takes the mirrored differences with
 // their signs turned, so a mirror-symmetric stencil gives L == R bitwise.  71 FP64 operations for 110 per variable,
-// 26 of them (products outside a fused multiply-add) as integers.
+// 26 of them (products outside a fused multiply-add) as integers (k_faces of 48 AMR-like blocks 4.77 -> 4.56 ms; the
+// same in the face physics, or in con2prim, cost more than it gave).
 __device__ __forceinline__ double weno_side64(double v2, double d0, double d1, double d2, double d3, double w0, double w1,
                                               double w2) {
   const double q0 = fma(-2.0, d0, mul64(5.0, d1)), q1 = fma(2.0, d2, d1), q2 = fma(4.0, d2, -d3);
@@ -822,7 +829,7 @@ struct C2PVal {
   bool vcap, eclamp;
 };
 
-// v^2 above its cap, eps below 0: FP64 without the FP64 pipe
+// a > b for b >= 0, a < 0: FP64 without the FP64 pipe
 __device__ __forceinline__ bool c2p_above(double a, double b) { return gtp64(a, b); }
 __device__ __forceinline__ bool c2p_above(float a, float b) { return a > b; }
 __device__ __forceinline__ bool c2p_neg(double a) { return neg64(a); }
@@ -848,7 +855,7 @@ __device__ __forceinline__ void c2p_master(R gam, R vmax2, const C2PInv<R>& I, R
   const R ge = R(1) + gam * E.eps;
   const R nuA = ge * E.iW;
   const R nuB = rdiv(ge * (R(1) + qm), R(1) + E.eps);
-  const R nu = nuA > nuB ? nuA : nuB;
+  const R nu = rmax(nuA, nuB);
   E.f = mu - rdiv(R(1), nu + mu * E.rbar2);
 }
 
@@ -877,7 +884,7 @@ __device__ __forceinline__ void c2p_master_fast(R gam, R vmax2, const C2PInv<R>&
   E.ed = d;
   const R G = d + gam * n;
   const R dn = d + n, q1 = R(1) + qm;
-  const bool a_wins = E.iW * dn > q1 * d;
+  const bool a_wins = rgt(E.iW * dn, q1 * d);
   const R P = a_wins ? E.iW : q1, Q = a_wins ? d : dn;
   E.f = mu - rdiv(Q, G * P + mu * E.rbar2 * Q);
 }
@@ -962,7 +969,7 @@ __device__ __forceinline__ void c2p_master_tab(const TabView<R>& t, R vmax2, con
   const R h = (R(1) + E.eps) + rdiv(E.p, E.rho);
   const R nuA = h * E.iW;
   const R nuB = rdiv(h * (R(1) + qm), R(1) + E.eps);
-  const R nu = nuA > nuB ? nuA : nuB;
+  const R nu = rmax(nuA, nuB);
   E.f = mu - rdiv(R(1), nu + mu * E.rbar2);
 }
 
@@ -982,14 +989,14 @@ __device__ __forceinline__ int illinois(Fn f, R a, R b, R fa, R fb, R tol, int m
                                         int* iters, bool* fresh = nullptr) {
   *iters = 0;
   if (fresh) *fresh = false;
-  if (fa == R(0)) { *root = a; *hi_out = a; return 0; }
-  if (fb == R(0)) { *root = b; *hi_out = b; return 0; }
-  if ((fa < R(0)) == (fb < R(0))) return -1;
+  if (rzero(fa)) { *root = a; *hi_out = a; return 0; }
+  if (rzero(fb)) { *root = b; *hi_out = b; return 0; }
+  if (c2p_neg(fa) == c2p_neg(fb)) return -1;
   int side = 0;
   for (int it = 1; it <= max_iter; ++it) {
     R c = rdiv(a * fb - b * fa, fb - fa);
-    if (!(c > a && c < b)) c = R(0.5) * (a + b);
-    if (!(c > a && c < b)) {
+    if (!(c2p_above(c, a) && c2p_above(b, c))) c = R(0.5) * (a + b);
+    if (!(c2p_above(c, a) && c2p_above(b, c))) {
       *root = c; *hi_out = b; *iters = it;
       if (fresh) *fresh = false;   // c itself was not evaluated
       return 0;
@@ -997,8 +1004,8 @@ __device__ __forceinline__ int illinois(Fn f, R a, R b, R fa, R fb, R tol, int m
     const R fc = f(c);
     *iters = it;
     if (fresh) *fresh = true;
-    if (fc == R(0)) { *root = c; *hi_out = c; return 0; }
-    if ((fc < R(0)) == (fa < R(0))) {
+    if (rzero(fc)) { *root = c; *hi_out = c; return 0; }
+    if (c2p_neg(fc) == c2p_neg(fa)) {
       a = c; fa = fc;
       if (side == -1) fb *= R(0.5);
       side = -1;
@@ -1007,7 +1014,7 @@ __device__ __forceinline__ int illinois(Fn f, R a, R b, R fa, R fb, R tol, int m
       if (side == +1) fa *= R(0.5);
       side = +1;
     }
-    if (b - a <= tol * c) { *root = c; *hi_out = b; return 0; }
+    if (!c2p_above(b - a, tol * c)) { *root = c; *hi_out = b; return 0; }
   }
   *hi_out = b;
   return -2;
@@ -1368,14 +1375,14 @@ __device__ __forceinline__ int con2prim_cell(const Site& site, const KParams& P,
           if (side == +1) fa *= 0.5;
           side = +1;
         }
-        if (b - a <= P.tol * mu) { root = mu; r = 0; fresh = true; break; }
+        if (!gtp64(b - a, P.tol * mu)) { root = mu; r = 0; fresh = true; break; }
         if (it >= P.max_iter) { r = -2; full = true; }
       } else if (phase == LO) {
         fa = fc; mu = b; phase = UP;
         continue;
       } else if (phase == UP) {
         fb = fc;
-        if (fa <= 0.0 && fb >= 0.0) start = true;
+        if ((neg64(fa) || zero64(fa)) && (gtp64(fb, 0.0) || zero64(fb))) start = true;
         else full = true;
       } else if (phase == Z) {
         fa = fc; a = 0.0; mu = b; phase = TOP;
@@ -1419,9 +1426,9 @@ __device__ __forceinline__ int con2prim_cell(const Site& site, const KParams& P,
         continue;
       }
       double c = div64(a * fb - b * fa, fb - fa);
-      if (!(c > a && c < b)) {
+      if (!(gtp64(c, a) && gtp64(b, c))) {
         c = 0.5 * (a + b);
-        if (!(c > a && c < b)) { root = c; r = 0; break; }   // c itself was not evaluated
+        if (!(gtp64(c, a) && gtp64(b, c))) { root = c; r = 0; break; }   // c itself was not evaluated
       }
       mu = c;
     }

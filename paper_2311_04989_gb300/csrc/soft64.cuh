@@ -131,6 +131,18 @@ __device__ __forceinline__ double rsqrt64(double x) {
   return from64(M + ((uint64_t)(uint32_t)(1021 - k) << 52));
 }
 
+// a * b by the FP64 pipe in a branch that is rarely taken: volatile, so that the compiler does not compute it
+// ahead of the branch for every thread
+__device__ __forceinline__ double mul_rare(double a, double b) {
+#ifdef __CUDACC__
+  double r;
+  asm volatile("mul.rn.f64 %0, %1, %2;" : "=d"(r) : "d"(a), "d"(b));
+  return r;
+#else
+  return a * b;
+#endif
+}
+
 // a * b, correctly rounded, for products of the hot FP64 kernels that are no part of a fused multiply-add: ~45
 // instructions of the idle issue slots for one of the FP64 pipe (70 cycles of a scheduler there).  Both
 // significands shifted to 64 bits, the product's upper 64 bits with the lower ones folded into the last, rounded
@@ -140,7 +152,7 @@ __device__ __forceinline__ double mul64(double a, double b) {
   const uint32_t ah = (uint32_t)(ua >> 32), bh = (uint32_t)(ub >> 32);
   const uint32_t ea = (ah >> 20) & 0x7ffu, eb = (bh >> 20) & 0x7ffu;
   const int e = (int)(ea + eb) - 1023;            // exponent of the product, or one more
-  if (!(ea - 1u < 2046u && eb - 1u < 2046u && (uint32_t)(e - 1) < 2044u)) return a * b;
+  if (!(ea - 1u < 2046u && eb - 1u < 2046u && (uint32_t)(e - 1) < 2044u)) return mul_rare(a, b);
   const uint32_t xh = 0x80000000u | fsr((uint32_t)ua, ah, 21), xl = (uint32_t)ua << 11;
   const uint32_t yh = 0x80000000u | fsr((uint32_t)ub, bh, 21), yl = (uint32_t)ub << 11;
   const uint64_t ll = mulw(xl, yl);
@@ -160,7 +172,7 @@ __device__ __forceinline__ double scale64(double x) {
   const uint64_t u = bits64(x);
   const uint32_t e = (uint32_t)(u >> 52) & 0x7ffu;
   if (e - (K + 1u) < 2046u - K) return from64(u - ((uint64_t)K << 52));
-  return x * (1.0 / (1 << K));
+  return mul_rare(x, 1.0 / (1 << K));
 }
 
 // whether x is finite, from the exponent bits of its high word (integer operations only: on GB300 an
