@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(kFT, 1) k_fused(const DBlock* __restrict__ blo
           } else {
             float src[6];
             CellMet<float> M;
-            cell_sources_at<float, EOS>(b, in, kp, i, j, pu, c, src, M);
+            cell_sources_at<float, EOS, 2>(b, in, kp, i, j, pu, c, src, M);
 #pragma unroll
             for (int v = 0; v < 5; ++v) {
               const int o = v * kFXY, oz = v * kFEA;

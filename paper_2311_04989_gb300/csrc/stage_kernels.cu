@@ -348,8 +348,14 @@ __device__ __forceinline__ void cell_gamma64(const DBlock& b, const InView<doubl
       const double* a = m.M[c] + v0;
       val[c] = 0.125 * (((a[0] + a[1]) + (a[sy] + a[sy + 1])) + ((a[sz] + a[sz + 1]) + (a[sz + sy] + a[sz + sy + 1])));
     }
-  } else {
-    cell_metric<double>(b, m, m.order, i, j, k, 4, 10, val, nullptr);
+  } else if (MODE == C2P_BRACKET || m.order == 2) {
+    cell_metric<double>(b, m, MODE == C2P_BRACKET ? m.order : 2, i, j, k, 4, 10, val, nullptr);
+  } else {   // one copy of the long interpolation, its results through local memory
+    double g4[6];
+#pragma unroll 1
+    for (int c = 0; c < 6; ++c) g4[c] = lagr_cell64(b, m.M[4 + c], b.vert, i, j, k);
+#pragma unroll
+    for (int c = 0; c < 6; ++c) val[4 + c] = g4[c];
   }
   c2pmet_from<MODE>(val + 4, M);
 }
@@ -370,12 +376,12 @@ __device__ __forceinline__ double accumulate_cell(const DBlock& b, const StateVi
 
 // U' of every conserved variable of interior cell (i, j, k): the geometric sources (cell_sources_at), then
 // accumulate_cell.  M: the cell metric, for the caller.
-template <class R, int EOS>
+template <class R, int EOS, int ORDER = 0>
 __device__ __forceinline__ void update_all(const DBlock& b, const InView<R>& in, const StateView& s,
                                            const Workspace& ws, const KParams& kp, int i, int j, int k,
                                            long long c, double q[6], CellMet<R>& M) {
   R src[6];
-  cell_sources_at<R, EOS>(b, in, kp, i, j, k, c, src, M);
+  cell_sources_at<R, EOS, ORDER>(b, in, kp, i, j, k, c, src, M);
   constexpr int NQ = EOS ? 6 : 5;
 #pragma unroll
   for (int v = 0; v < NQ; ++v) q[v] = accumulate_cell<R>(b, s, ws, kp, i, j, k, c, v, src[v]);
@@ -488,11 +494,11 @@ __device__ __forceinline__ Job job_cell(const DBlock& b, int e) {
   return o;
 }
 
-// k_jobs<EOS>: U' of the queued cells of the mixed stage (update_all on the FP32 inputs) into Uo.  A kernel of
+// k_jobs<EOS, ORDER>: U' of the queued cells of the mixed stage (update_all on the FP32 inputs) into Uo.  A kernel of
 // its own: with con2prim in the same one, its registers and code kept the solve at 12 warps per SM and out of
 // the instruction cache (AMR-like batch, 256 blocks, 4.3 M cells: 3.40 ms together, 2.70 ms as two kernels at
 // 96 registers; at 80 2.79, at 128 2.77, at 168 3.02).  0.62 ms there, latency-bound.
-template <int EOS>
+template <int EOS, int ORDER>
 __global__ void __maxnreg__(96) k_jobs(const DBlock* __restrict__ blocks, const __grid_constant__ InView<float> in,
                        const __grid_constant__ StateView s, const __grid_constant__ Workspace ws,
                        const __grid_constant__ KParams kp) {
@@ -503,7 +509,7 @@ __global__ void __maxnreg__(96) k_jobs(const DBlock* __restrict__ blocks, const 
     const Job o = job_cell(b, job.y);
     double q[6];
     CellMet<float> M32;
-    update_all<float, EOS>(b, in, s, ws, kp, o.i, o.j, o.k, o.c, q, M32);
+    update_all<float, EOS, ORDER>(b, in, s, ws, kp, o.i, o.j, o.k, o.c, q, M32);
 #pragma unroll
     for (int v = 0; v < (EOS ? 6 : 5); ++v) s.Uo[v][o.c] = q[v];
   }
@@ -886,7 +892,10 @@ static cudaError_t stage_impl(const DBlock* blocks, const KLaunch kl[SK_N], cons
     KLaunch qq = q;
     qq.nwork = (q.nwork + q.threads - 1) / q.threads;   // q.nwork = the number of interior cells
     constexpr bool mixed = sizeof(R) == sizeof(float);
-    if constexpr (mixed) k_jobs<EOS><<<stage_grid(k_jobs<EOS>, qq, 0), q.threads, 0, st>>>(blocks, in, s, ws, kp);
+    if constexpr (mixed) {
+      if (in.order == 4) k_jobs<EOS, 4><<<stage_grid(k_jobs<EOS, 4>, qq, 0), q.threads, 0, st>>>(blocks, in, s, ws, kp);
+      else k_jobs<EOS, 2><<<stage_grid(k_jobs<EOS, 2>, qq, 0), q.threads, 0, st>>>(blocks, in, s, ws, kp);
+    }
     launch_c2p<EOS, mixed>(blocks, qq, in64, s, ws, kp, st);
   }
   if (ev) cudaEventRecord(ev[7], st);

@@ -64,13 +64,15 @@ __device__ __forceinline__ double accumulate_vals(const DBlock& b, const StateVi
 // Geometric sources src[0..5] of interior cell (i, j, k) (none for D and D Y_e) in R from the stage-input
 // metric (vertex interpolant: values and first derivatives), primitives and mean densitised face field;
 // M: the cell metric, for the caller.
-template <class R, int EOS>
+// ORDER: the metric's interpolation order where it is known at compile time, else 0
+template <class R, int EOS, int ORDER = 0>
 __device__ __forceinline__ void cell_sources_at(const DBlock& b, const InView<R>& in, const KParams& kp, int i, int j,
                                                 int k, long long c, R src[6], CellMet<R>& M) {
   const bool kzero = in.k_zero != 0;
   R val[16], dm[3][10];
-  cell_metric<R>(b, in, in.order, i, j, k, 0, 10, val, dm);
-  if (!kzero) cell_metric<R>(b, in, in.order, i, j, k, 10, 16, val, nullptr);
+  const int order = ORDER ? ORDER : in.order;
+  cell_metric<R>(b, in, order, i, j, k, 0, 10, val, dm);
+  if (!kzero) cell_metric<R>(b, in, order, i, j, k, 10, 16, val, nullptr);
   cellmet_from<R>(val, kzero, M);
   R wv[6], Bd[3];
 #pragma unroll
