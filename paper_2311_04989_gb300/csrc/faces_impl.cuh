@@ -88,6 +88,7 @@ __global__ void __maxnreg__(sizeof(R) == sizeof(float) ? (EOS == GR_EOS_TABLE ? 
                                                     int nwork, const __grid_constant__ InView<R> in,
                                                     const __grid_constant__ Workspace ws,
                                                     const __grid_constant__ KParams kp) {
+  stage_begin();
   for (int it = blockIdx.x; it < nwork; it += gridDim.x) {
     const Work w = work[it];
     const DBlock b = blocks[w.block];
@@ -100,20 +101,19 @@ __global__ void __maxnreg__(sizeof(R) == sizeof(float) ? (EOS == GR_EOS_TABLE ? 
 
 template <class R, int EOS, int METHOD>
 static cudaError_t launch_faces_m(const KLaunch& f, const DBlock* blocks, const InView<R>& in, const Workspace& ws,
-                                  const KParams& kp, cudaStream_t st) {
-  k_faces<R, EOS, METHOD><<<stage_grid(k_faces<R, EOS, METHOD>, f, 0), f.threads, 0, st>>>(blocks, f.work, f.nwork,
-                                                                                          in, ws, kp);
-  return cudaGetLastError();
+                                  const KParams& kp, cudaStream_t st, bool overlap) {
+  return launch_stage_kernel(overlap, k_faces<R, EOS, METHOD>, stage_grid(k_faces<R, EOS, METHOD>, f, 0), f.threads, 0, st,
+                             blocks, f.work, f.nwork, in, ws, kp);
 }
 
 template <class R, int EOS>
 static cudaError_t launch_faces_e(const KLaunch& f, const DBlock* blocks, const InView<R>& in, const Workspace& ws,
-                                  const KParams& kp, cudaStream_t st) {
+                                  const KParams& kp, cudaStream_t st, bool overlap) {
   switch (kp.recon) {
-    case GR_RECON_PLM: return launch_faces_m<R, EOS, GR_RECON_PLM>(f, blocks, in, ws, kp, st);
-    case GR_RECON_WENO5: return launch_faces_m<R, EOS, GR_RECON_WENO5>(f, blocks, in, ws, kp, st);
-    case GR_RECON_PPM: return launch_faces_m<R, EOS, GR_RECON_PPM>(f, blocks, in, ws, kp, st);
-    default: return launch_faces_m<R, EOS, GR_RECON_WENOZ>(f, blocks, in, ws, kp, st);
+    case GR_RECON_PLM: return launch_faces_m<R, EOS, GR_RECON_PLM>(f, blocks, in, ws, kp, st, overlap);
+    case GR_RECON_WENO5: return launch_faces_m<R, EOS, GR_RECON_WENO5>(f, blocks, in, ws, kp, st, overlap);
+    case GR_RECON_PPM: return launch_faces_m<R, EOS, GR_RECON_PPM>(f, blocks, in, ws, kp, st, overlap);
+    default: return launch_faces_m<R, EOS, GR_RECON_WENOZ>(f, blocks, in, ws, kp, st, overlap);
   }
 }
 
@@ -122,8 +122,8 @@ static cudaError_t launch_faces_e(const KLaunch& f, const DBlock* blocks, const 
 #define GRS_DEFINE_LAUNCH_FACES(R)                                                                        \
   namespace grs {                                                                                        \
   cudaError_t launch_faces(const KLaunch& f, const DBlock* blocks, const InView<R>& in, const Workspace& ws, \
-                           const KParams& kp, cudaStream_t st) {                                        \
-    return kp.eos == GR_EOS_TABLE ? launch_faces_e<R, GR_EOS_TABLE>(f, blocks, in, ws, kp, st)           \
-                                  : launch_faces_e<R, GR_EOS_IDEAL>(f, blocks, in, ws, kp, st);          \
+                           const KParams& kp, cudaStream_t st, bool overlap) {                                        \
+    return kp.eos == GR_EOS_TABLE ? launch_faces_e<R, GR_EOS_TABLE>(f, blocks, in, ws, kp, st, overlap)           \
+                                  : launch_faces_e<R, GR_EOS_IDEAL>(f, blocks, in, ws, kp, st, overlap);          \
   }                                                                                                      \
   }

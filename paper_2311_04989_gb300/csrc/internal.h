@@ -214,11 +214,12 @@ struct KLaunch {
   int persistent;
 };
 
-// k_faces launchers (faces_f32.cu, faces_f64.cu): one instantiation per EOS and reconstruction method
+// k_faces launchers (faces_f32.cu, faces_f64.cu): one instantiation per EOS and reconstruction method; overlap:
+// its launch may overlap the previous kernel (stage_common.cuh)
 cudaError_t launch_faces(const KLaunch& f, const DBlock* blocks, const InView<float>& in, const Workspace& ws,
-                         const KParams& kp, cudaStream_t st);
+                         const KParams& kp, cudaStream_t st, bool overlap);
 cudaError_t launch_faces(const KLaunch& f, const DBlock* blocks, const InView<double>& in, const Workspace& ws,
-                         const KParams& kp, cudaStream_t st);
+                         const KParams& kp, cudaStream_t st, bool overlap);
 
 // Fused sweep of the mixed path (fused.cu): faces, corner EMFs, CT and the update of every block in one
 // launch (one CTA per block); the blocks must satisfy fused_block_ok (ghost width 3, at most 16 x 16 cells

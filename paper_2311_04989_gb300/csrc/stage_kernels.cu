@@ -44,6 +44,7 @@ struct CastList {
 };
 
 __global__ void __launch_bounds__(256) k_cast(const __grid_constant__ CastList L) {
+  stage_begin();
   const int seg = blockIdx.y;
   if (seg >= L.count) return;
   const double* __restrict__ s = L.src[seg];
@@ -102,6 +103,14 @@ __device__ __forceinline__ void cellprep_cell(const DBlock& b, const InView<R>& 
   }
 }
 
+// the stage's counters, for the kernels after this one: no con2prim jobs, no block with a large flux (on a refined
+// mesh, whose coarse fluxes the level fix rewrites, every block)
+__device__ __forceinline__ void stage_reset(const Workspace& ws) {
+  if (blockIdx.x != 0) return;
+  if (threadIdx.x == 0) *ws.njobs = 0;
+  for (int b = threadIdx.x; b < ws.nfbad; b += blockDim.x) ws.fbad[b] = ws.nlvl ? 1 : 0;
+}
+
 template <class R>
 __device__ __forceinline__ void cellprep_body(const Work& w, const DBlock& b, const InView<R>& in,
                                               const Workspace& ws) {
@@ -123,6 +132,8 @@ template <class R>
 __global__ void __launch_bounds__(kMaxTile) k_cellprep(const DBlock* __restrict__ blocks, const Work* __restrict__ work,
                                                        int nwork, const __grid_constant__ InView<R> in,
                                                        const __grid_constant__ Workspace ws) {
+  stage_begin();
+  stage_reset(ws);
   for (int it = blockIdx.x; it < nwork; it += gridDim.x) {
     const Work w = work[it];
     cellprep_body<R>(w, blocks[w.block], in, ws);
@@ -149,6 +160,8 @@ __global__ void __launch_bounds__(kSweepThreads) k_cellprep_sweep(const DBlock* 
                                                                   const __grid_constant__ InView<R> in,
                                                                   const __grid_constant__ Workspace ws) {
   extern __shared__ __align__(16) unsigned char sweep_smem[];
+  stage_begin();
+  stage_reset(ws);
   R* sm = reinterpret_cast<R*>(sweep_smem);   // [buffer 2][component 10][kSweepVerts]
   const SweepWork w = work[blockIdx.x];
   const DBlock b = blocks[w.block];
@@ -213,7 +226,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_cellprep_sweep(const DBlock* 
 
 template <class R>
 static cudaError_t launch_cellprep_sweep(const DBlock* blocks, const InView<R>& in, const Workspace& ws,
-                                         cudaStream_t st) {
+                                         cudaStream_t st, bool overlap) {
   constexpr size_t smem = sizeof(R) * 2 * 10 * kSweepVerts;
   // above the default 48 KB: the opt-in is per device (set once on each, one bit per device)
   static unsigned long long attr = 0;
@@ -223,8 +236,7 @@ static cudaError_t launch_cellprep_sweep(const DBlock* blocks, const InView<R>& 
     if (e != cudaSuccess) return e;
     attr |= 1ull << dev;
   }
-  k_cellprep_sweep<R><<<ws.nsweep, kSweepThreads, smem, st>>>(blocks, ws.sweep, in, ws);
-  return cudaGetLastError();
+  return launch_stage_kernel(overlap, k_cellprep_sweep<R>, ws.nsweep, kSweepThreads, smem, st, blocks, ws.sweep, in, ws);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -269,6 +281,7 @@ template <class R>
 __global__ void __launch_bounds__(kMaxTile) k_edges(const DBlock* __restrict__ blocks, const Work* __restrict__ work,
                                                     int nwork, const __grid_constant__ Workspace ws,
                                                     const __grid_constant__ KParams kp) {
+  stage_begin();
   for (int it = blockIdx.x; it < nwork; it += gridDim.x) {
     const Work w = work[it];
     const DBlock b = blocks[w.block];
@@ -324,6 +337,7 @@ __global__ void __launch_bounds__(kMaxTile) k_ct(const DBlock* __restrict__ bloc
                                                  int nwork, const __grid_constant__ StateView s,
                                                  const __grid_constant__ Workspace ws,
                                                  const __grid_constant__ KParams kp) {
+  stage_begin();
   switch (kp.rk_form) {   // uniform over the grid: one branch, taken once
     case 0: ct_loop<R, 0>(blocks, work, nwork, s, ws, kp); break;
     case RK_G0: ct_loop<R, RK_G0>(blocks, work, nwork, s, ws, kp); break;
@@ -465,6 +479,7 @@ __global__ void __launch_bounds__(kMaxTile, sizeof(R) == sizeof(float) ? 4 : 0) 
                                                      const __grid_constant__ StateView s,
                                                      const __grid_constant__ Workspace ws,
                                                      const __grid_constant__ KParams kp) {
+  stage_begin();
   const unsigned lane = threadIdx.x & 31u;
   for (int it = blockIdx.x; it < nwork; it += gridDim.x) {
     const Work w = work[it];
@@ -502,6 +517,7 @@ template <int EOS, int ORDER>
 __global__ void __maxnreg__(96) k_jobs(const DBlock* __restrict__ blocks, const __grid_constant__ InView<float> in,
                        const __grid_constant__ StateView s, const __grid_constant__ Workspace ws,
                        const __grid_constant__ KParams kp) {
+  stage_begin();
   const int n = *ws.njobs;
   for (int jdx = blockIdx.x * blockDim.x + threadIdx.x; jdx < n; jdx += gridDim.x * blockDim.x) {
     const int2 job = ws.jobs[jdx];
@@ -549,6 +565,7 @@ template <int EOS, int MODE>
 __global__ void __maxnreg__(MODE == C2P_NEWTON ? 96 : 128) k_c2p(const DBlock* __restrict__ blocks, const __grid_constant__ InView<double> in64,
                                        const __grid_constant__ StateView s, const __grid_constant__ Workspace ws,
                                        const __grid_constant__ KParams kp) {
+  stage_begin();
   const int n = *ws.njobs;
   for (int jdx = blockIdx.x * blockDim.x + threadIdx.x; jdx < n; jdx += gridDim.x * blockDim.x) {
     const int2 job = ws.jobs[jdx];
@@ -801,16 +818,16 @@ cudaError_t launch_cast_pool(const double* src, float* dst, long long n, cudaStr
 // con2prim of the queued cells of a stage
 template <int EOS, int MODE>
 static void launch_c2p_m(const DBlock* blocks, const KLaunch& q, const InView<double>& in64, const StateView& s,
-                         const Workspace& ws, const KParams& kp, cudaStream_t st) {
-  k_c2p<EOS, MODE><<<stage_grid(k_c2p<EOS, MODE>, q, 0), q.threads, 0, st>>>(blocks, in64, s, ws, kp);
+                         const Workspace& ws, const KParams& kp, cudaStream_t st, bool overlap) {
+  launch_stage_kernel(overlap, k_c2p<EOS, MODE>, stage_grid(k_c2p<EOS, MODE>, q, 0), q.threads, 0, st, blocks, in64, s, ws, kp);
 }
 template <int EOS, bool MIXED>
 static void launch_c2p(const DBlock* blocks, const KLaunch& q, const InView<double>& in64, const StateView& s,
-                       const Workspace& ws, const KParams& kp, cudaStream_t st) {
-  if constexpr (!MIXED) launch_c2p_m<EOS, C2P_PLAIN>(blocks, q, in64, s, ws, kp, st);
+                       const Workspace& ws, const KParams& kp, cudaStream_t st, bool overlap) {
+  if constexpr (!MIXED) launch_c2p_m<EOS, C2P_PLAIN>(blocks, q, in64, s, ws, kp, st, overlap);
   else if (kp.c2p_guess == GR_GUESS_FP32 || (kp.c2p_guess == GR_GUESS_NONE && !kp.dt_dev))
-    launch_c2p_m<EOS, C2P_NEWTON>(blocks, q, in64, s, ws, kp, st);
-  else launch_c2p_m<EOS, C2P_BRACKET>(blocks, q, in64, s, ws, kp, st);
+    launch_c2p_m<EOS, C2P_NEWTON>(blocks, q, in64, s, ws, kp, st, overlap);
+  else launch_c2p_m<EOS, C2P_BRACKET>(blocks, q, in64, s, ws, kp, st, overlap);
 }
 
 // The mixed stage through the fused sweep: cell prep, k_fused (faces, EMFs, CT, update), con2prim of the
@@ -818,7 +835,7 @@ static void launch_c2p(const DBlock* blocks, const KLaunch& q, const InView<doub
 static cudaError_t stage_fused(const DBlock* blocks, int nblocks, const KLaunch kl[SK_N], const InView<float>& in,
                                const InView<double>& in64, const StateView& s, const Workspace& ws, const KParams& kp,
                                cudaStream_t st, cudaEvent_t* ev) {
-  cudaError_t e = launch_cellprep_sweep<float>(blocks, in, ws, st);
+  cudaError_t e = launch_cellprep_sweep<float>(blocks, in, ws, st, false);
   if (e != cudaSuccess) return e;
   if (ev) cudaEventRecord(ev[2], st);
   e = cudaMemsetAsync(ws.njobs, 0, sizeof(int), st);
@@ -832,7 +849,7 @@ static cudaError_t stage_fused(const DBlock* blocks, int nblocks, const KLaunch 
   if (q.nwork) {
     KLaunch qq = q;
     qq.nwork = (q.nwork + q.threads - 1) / q.threads;
-    launch_c2p<GR_EOS_IDEAL, true>(blocks, qq, in64, s, ws, kp, st);
+    launch_c2p<GR_EOS_IDEAL, true>(blocks, qq, in64, s, ws, kp, st, false);
   }
   if (ev) cudaEventRecord(ev[7], st);
   return cudaGetLastError();
@@ -841,35 +858,34 @@ static cudaError_t stage_fused(const DBlock* blocks, int nblocks, const KLaunch 
 template <class R, int EOS>
 static cudaError_t stage_impl(const DBlock* blocks, const KLaunch kl[SK_N], const InView<R>& in,
                               const InView<double>& in64, const StateView& s, const Workspace& ws, const KParams& kp,
-                              cudaStream_t st, cudaEvent_t* ev) {
+                              cudaStream_t st, cudaEvent_t* ev, bool after_cast) {
+  const bool overlap = ev == nullptr;   // events between the kernels order them fully
   const KLaunch& a = kl[SK_CELLPREP];
   if (in.order == 2 && ws.nsweep) {   // the order-2 metric: the z sweep (same results, any launch shape)
-    const cudaError_t es = launch_cellprep_sweep<R>(blocks, in, ws, st);
+    const cudaError_t es = launch_cellprep_sweep<R>(blocks, in, ws, st, overlap && after_cast);
     if (es != cudaSuccess) return es;
   } else if (a.nwork) {
-    k_cellprep<R><<<stage_grid(k_cellprep<R>, a, 0), a.threads, 0, st>>>(blocks, a.work, a.nwork, in, ws);
+    launch_stage_kernel(overlap && after_cast, k_cellprep<R>, stage_grid(k_cellprep<R>, a, 0), a.threads, 0, st, blocks,
+                        a.work, a.nwork, in, ws);
   }
   if (ev) cudaEventRecord(ev[2], st);
   const KLaunch& f = kl[SK_FACES];
-  if constexpr (sizeof(R) == sizeof(float)) {   // the per-block flux flags: set for all on a refined mesh
-    const cudaError_t eb = cudaMemsetAsync(ws.fbad, ws.nlvl ? 1 : 0, ws.nfbad, st);
-    if (eb != cudaSuccess) return eb;
-  }
   if constexpr (sizeof(R) == sizeof(float) && EOS == GR_EOS_IDEAL) {
     if (ws.nftiles > 0 && in.order == 2) {   // the tiled face sweep (the host checked that every block qualifies)
       const cudaError_t e = launch_faces_tile(blocks, ws.ftiles, ws.nftiles, in, ws, kp, st);
       if (e != cudaSuccess) return e;
     } else if (f.nwork) {
-      const cudaError_t e = launch_faces(f, blocks, in, ws, kp, st);
+      const cudaError_t e = launch_faces(f, blocks, in, ws, kp, st, overlap);
       if (e != cudaSuccess) return e;
     }
   } else if (f.nwork) {
-    const cudaError_t e = launch_faces(f, blocks, in, ws, kp, st);
+    const cudaError_t e = launch_faces(f, blocks, in, ws, kp, st, overlap);
     if (e != cudaSuccess) return e;
   }
   if (ev) cudaEventRecord(ev[3], st);
   const KLaunch& e = kl[SK_EDGES];
-  if (e.nwork) k_edges<R><<<stage_grid(k_edges<R>, e, 0), e.threads, 0, st>>>(blocks, e.work, e.nwork, ws, kp);
+  if (e.nwork)
+    launch_stage_kernel(overlap, k_edges<R>, stage_grid(k_edges<R>, e, 0), e.threads, 0, st, blocks, e.work, e.nwork, ws, kp);
   if (ws.nlvl) {   // refined mesh: coarse fluxes and EMFs on level boundaries from the fine ones
     const cudaError_t el = launch_level_fix(sizeof(R) == sizeof(float) ? GR_PREC_MIXED : GR_PREC_FP64, blocks, ws.lvl,
                                             ws.nlvl, ws, EOS == GR_EOS_TABLE, st);
@@ -877,13 +893,13 @@ static cudaError_t stage_impl(const DBlock* blocks, const KLaunch kl[SK_N], cons
   }
   if (ev) cudaEventRecord(ev[4], st);
   const KLaunch& c = kl[SK_CT];
-  if (c.nwork) k_ct<R><<<stage_grid(k_ct<R>, c, 0), c.threads, 0, st>>>(blocks, c.work, c.nwork, s, ws, kp);
+  if (c.nwork)
+    launch_stage_kernel(overlap, k_ct<R>, stage_grid(k_ct<R>, c, 0), c.threads, 0, st, blocks, c.work, c.nwork, s, ws, kp);
   if (ev) cudaEventRecord(ev[5], st);
   const KLaunch& u = kl[SK_UPDATE];
-  cudaError_t e0 = cudaMemsetAsync(ws.njobs, 0, sizeof(int), st);
-  if (e0 != cudaSuccess) return e0;
   if (u.nwork)
-    k_update<R, EOS><<<stage_grid(k_update<R, EOS>, u, 0), u.threads, 0, st>>>(blocks, u.work, u.nwork, in, s, ws, kp);
+    launch_stage_kernel(overlap, k_update<R, EOS>, stage_grid(k_update<R, EOS>, u, 0), u.threads, 0, st, blocks, u.work,
+                        u.nwork, in, s, ws, kp);
   if (ev) cudaEventRecord(ev[6], st);
   // the job count is known only on the device: one CTA per possible job (the rest exit at once), or
   // a persistent grid that strides over the list
@@ -893,10 +909,12 @@ static cudaError_t stage_impl(const DBlock* blocks, const KLaunch kl[SK_N], cons
     qq.nwork = (q.nwork + q.threads - 1) / q.threads;   // q.nwork = the number of interior cells
     constexpr bool mixed = sizeof(R) == sizeof(float);
     if constexpr (mixed) {
-      if (in.order == 4) k_jobs<EOS, 4><<<stage_grid(k_jobs<EOS, 4>, qq, 0), q.threads, 0, st>>>(blocks, in, s, ws, kp);
-      else k_jobs<EOS, 2><<<stage_grid(k_jobs<EOS, 2>, qq, 0), q.threads, 0, st>>>(blocks, in, s, ws, kp);
+      if (in.order == 4)
+        launch_stage_kernel(overlap, k_jobs<EOS, 4>, stage_grid(k_jobs<EOS, 4>, qq, 0), q.threads, 0, st, blocks, in, s, ws, kp);
+      else
+        launch_stage_kernel(overlap, k_jobs<EOS, 2>, stage_grid(k_jobs<EOS, 2>, qq, 0), q.threads, 0, st, blocks, in, s, ws, kp);
     }
-    launch_c2p<EOS, mixed>(blocks, qq, in64, s, ws, kp, st);
+    launch_c2p<EOS, mixed>(blocks, qq, in64, s, ws, kp, st, overlap);
   }
   if (ev) cudaEventRecord(ev[7], st);
   return cudaGetLastError();
@@ -914,12 +932,13 @@ cudaError_t launch_stage(int precision, const DBlock* blocks, const KLaunch kl[S
     if (ev) cudaEventRecord(ev[1], st);
     const InView<float> in32 = view32(m, s, sh);
     if (nfused > 0 && !tab) return stage_fused(blocks, nfused, kl, in32, in64, s, ws, kp, st, ev);
-    return tab ? stage_impl<float, GR_EOS_TABLE>(blocks, kl, in32, in64, s, ws, kp, st, ev)
-               : stage_impl<float, GR_EOS_IDEAL>(blocks, kl, in32, in64, s, ws, kp, st, ev);
+    const bool cast = !s.W32[0] || (cast_metric && !m.v32[0]);
+    return tab ? stage_impl<float, GR_EOS_TABLE>(blocks, kl, in32, in64, s, ws, kp, st, ev, cast)
+               : stage_impl<float, GR_EOS_IDEAL>(blocks, kl, in32, in64, s, ws, kp, st, ev, cast);
   }
   if (ev) cudaEventRecord(ev[1], st);
-  return tab ? stage_impl<double, GR_EOS_TABLE>(blocks, kl, in64, in64, s, ws, kp, st, ev)
-             : stage_impl<double, GR_EOS_IDEAL>(blocks, kl, in64, in64, s, ws, kp, st, ev);
+  return tab ? stage_impl<double, GR_EOS_TABLE>(blocks, kl, in64, in64, s, ws, kp, st, ev, false)
+             : stage_impl<double, GR_EOS_IDEAL>(blocks, kl, in64, in64, s, ws, kp, st, ev, false);
 }
 
 cudaError_t launch_prim2con(const DBlock* blocks, const Work* work, int nwork, const MetricView& m,
