@@ -178,16 +178,30 @@ struct AdmVertArgs {
   double* out[10];
 };
 
-// midpoint weights of the 2- and 4-point Lagrange interpolants
+// midpoint weights of the 2- and 4-point Lagrange interpolants (FP32)
 template <class R, int NP> __device__ __forceinline__ R mid_weight(int s);
-template <> __device__ __forceinline__ double mid_weight<double, 2>(int) { return 0.5; }
 template <> __device__ __forceinline__ float mid_weight<float, 2>(int) { return 0.5f; }
-template <> __device__ __forceinline__ double mid_weight<double, 4>(int s) {
-  return (s == 1 || s == 2) ? 9.0 / 16 : -1.0 / 16;
-}
 template <> __device__ __forceinline__ float mid_weight<float, 4>(int s) {
   return (s == 1 || s == 2) ? 9.0f / 16 : -1.0f / 16;
 }
+
+// One axis of the interpolant at a vertex from its NP cells, stride `st` apart.  FP64: the weights times 2 or 16 per
+// axis (1, 1 or -1, 9, 9, -1), so that an order-4 axis takes three FP64 instructions for four and an order-2 one one
+// for two; axis_end takes the powers of two off at the end, exactly.
+template <class R, int NP>
+__device__ __forceinline__ R axis_sum(const R* src, size_t st) {
+  if constexpr (sizeof(R) == sizeof(double)) {
+    if constexpr (NP == 2) return src[0] + src[st];
+    else return fma(R(9), src[st] + src[2 * st], -(src[0] + src[3 * st]));
+  } else {
+    R s = 0;
+#pragma unroll
+    for (int q = 0; q < NP; ++q) s = fma(mid_weight<R, NP>(q), src[q * st], s);
+    return s;
+  }
+}
+template <int NP> __device__ __forceinline__ double axis_end(double s) { return scale64<NP == 2 ? 3 : 12>(s); }
+template <int NP> __device__ __forceinline__ double axis_end(float s) { return to64(s); }
 
 // Work: block, dir = number of vertex planes Z of the slab, start = first vertex plane z0.
 // Vertex v along an axis lies between cells v-1 and v; its NP-point stencil is cells v-r .. v+r-1,
@@ -221,21 +235,13 @@ __global__ void __launch_bounds__(kAdmThreads) k_adm_verts(const DBlock* __restr
   const int nx = V0 * C1 * CZ;
   Walk3 wx((int)threadIdx.x, kAdmThreads, V0, C1);
   for (int t = threadIdx.x; t < nx; t += kAdmThreads, wx.step()) {
-    const R* src = A + ((size_t)wx.z * C1 + wx.y) * C0 + wx.x;
-    R s = 0;
-#pragma unroll
-    for (int q = 0; q < NP; ++q) s = fma(mid_weight<R, NP>(q), src[q], s);
-    X[t] = s;
+    X[t] = axis_sum<R, NP>(A + ((size_t)wx.z * C1 + wx.y) * C0 + wx.x, 1);
   }
   __syncthreads();
   const int ny = V0 * V1 * CZ;
   Walk3 wy((int)threadIdx.x, kAdmThreads, V0, V1);
   for (int t = threadIdx.x; t < ny; t += kAdmThreads, wy.step()) {
-    const R* src = X + ((size_t)wy.z * C1 + wy.y) * V0 + wy.x;
-    R s = 0;
-#pragma unroll
-    for (int q = 0; q < NP; ++q) s = fma(mid_weight<R, NP>(q), src[(size_t)q * V0], s);
-    A[t] = s;
+    A[t] = axis_sum<R, NP>(X + ((size_t)wy.z * C1 + wy.y) * V0 + wy.x, V0);
   }
   __syncthreads();
   double* __restrict__ out = a.out[blockIdx.y];
@@ -243,11 +249,8 @@ __global__ void __launch_bounds__(kAdmThreads) k_adm_verts(const DBlock* __restr
   Walk3 wz((int)threadIdx.x, kAdmThreads, V0, V1);
   for (int t = threadIdx.x; t < nz; t += kAdmThreads, wz.step()) {
     const int vi = wz.x, vj = wz.y, vk = wz.z;
-    const R* src = A + ((size_t)vk * V1 + vj) * V0 + vi;
-    R s = 0;
-#pragma unroll
-    for (int q = 0; q < NP; ++q) s = fma(mid_weight<R, NP>(q), src[(size_t)q * V0 * V1], s);
-    out[b.vert + vix(b, vi, vj, z0 + vk)] = to64(s);
+    out[b.vert + vix(b, vi, vj, z0 + vk)] =
+        axis_end<NP>(axis_sum<R, NP>(A + ((size_t)vk * V1 + vj) * V0 + vi, (size_t)V0 * V1));
   }
 }
 
