@@ -41,9 +41,9 @@ __device__ __forceinline__ float fdiv(float a, float b) {
   asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
   return y;
 }
-// a/b: IEEE division in FP64; the fast approximate FP32 division (2 ulp) on the mixed path, fdiv but for the
-// face and cell physics with a table, where it changes which products the compiler fuses (and the FP32 fluxes by
-// their rounding)
+// a/b: IEEE division in FP64; the fast approximate FP32 division (2 ulp) on the mixed path, fdiv but with a table:
+// there it changes which products the compiler fuses, the FP32 fluxes by their rounding, and the pre-solve's bracket
+// (and with it the status bit of a rejected one)
 template <class R, int EOS = GR_EOS_IDEAL>
 __device__ __forceinline__ R rdiv(R a, R b) {
   if constexpr (sizeof(R) == sizeof(double)) return div64(a, b);
@@ -1005,7 +1005,7 @@ __device__ __forceinline__ float c2p_slope32(float gam, float vmax2, const C2PIn
 template <class R>
 __device__ __forceinline__ void c2p_master_tab(const TabView<R>& t, R vmax2, const C2PInv<R>& I, R mu,
                                                C2PVal<R>& E, int* khint) {
-  E.x = rdiv(R(1), R(1) + mu * I.b2);
+  E.x = rdiv<R, GR_EOS_TABLE>(R(1), R(1) + mu * I.b2);
   E.rbar2 = E.x * E.x * I.r2 + mu * E.x * (R(1) + E.x) * I.rb * I.rb;
   const R qbar = I.q - R(0.5) * I.b2 - R(0.5) * mu * mu * E.x * E.x * (I.b2 * I.r2 - I.rb * I.rb);
   E.v2 = mu * mu * E.rbar2;
@@ -1013,7 +1013,7 @@ __device__ __forceinline__ void c2p_master_tab(const TabView<R>& t, R vmax2, con
   if (E.vcap) E.v2 = vmax2;
   E.iW = sqrt_r(R(1) - E.v2);
   const R qm = qbar - mu * E.rbar2;
-  E.eps = rdiv(qm * (R(1) + E.iW) + E.v2, E.iW * (R(1) + E.iW));
+  E.eps = rdiv<R, GR_EOS_TABLE>(qm * (R(1) + E.iW) + E.v2, E.iW * (R(1) + E.iW));
   E.rho = I.D * E.iW;
   E.eclamp = false;
   bool cl = false;
@@ -1027,25 +1027,25 @@ __device__ __forceinline__ void c2p_master_tab(const TabView<R>& t, R vmax2, con
   *khint = k;
   if (cl) { E.eps = rexpm1(tab_T(t, t.f[1], L, k, wT)); E.eclamp = true; }
   E.p = E.rho * rexp(tab_T(t, t.f[0], L, k, wT));
-  const R h = (R(1) + E.eps) + rdiv(E.p, E.rho);
+  const R h = (R(1) + E.eps) + rdiv<R, GR_EOS_TABLE>(E.p, E.rho);
   const R nuA = h * E.iW;
-  const R nuB = rdiv(h * (R(1) + qm), R(1) + E.eps);
+  const R nuB = rdiv<R, GR_EOS_TABLE>(h * (R(1) + qm), R(1) + E.eps);
   const R nu = rmax(nuA, nuB);
-  E.f = mu - rdiv(R(1), nu + mu * E.rbar2);
+  E.f = mu - rdiv<R, GR_EOS_TABLE>(R(1), nu + mu * E.rbar2);
 }
 
 // Auxiliary function mu sqrt(h0^2 + rbar^2(mu)) - 1 whose root bounds the master root from above;
 // h0 = minimum enthalpy of the EOS (1 for the ideal gas), passed squared
-template <class R>
+template <class R, int EOS>
 __device__ __forceinline__ R c2p_aux(const C2PInv<R>& I, R h0sq, R mu) {
-  const R x = rdiv(R(1), R(1) + mu * I.b2);
+  const R x = rdiv<R, EOS>(R(1), R(1) + mu * I.b2);
   const R rbar2 = x * x * I.r2 + mu * x * (R(1) + x) * I.rb * I.rb;
   return mu * sqrt_r(h0sq + rbar2) - R(1);
 }
 
 // Illinois on [a,b] (f(a) < 0 < f(b) or reverse).  Returns 0 (root), -1 (no sign change), -2 (cap).
 // *fresh (optional): whether the root is the point f was last evaluated at.
-template <class R, class Fn>
+template <class R, int EOS, class Fn>
 __device__ __forceinline__ int illinois(Fn f, R a, R b, R fa, R fb, R tol, int max_iter, R* root, R* hi_out,
                                         int* iters, bool* fresh = nullptr) {
   *iters = 0;
@@ -1055,7 +1055,7 @@ __device__ __forceinline__ int illinois(Fn f, R a, R b, R fa, R fb, R tol, int m
   if (c2p_neg(fa) == c2p_neg(fb)) return -1;
   int side = 0;
   for (int it = 1; it <= max_iter; ++it) {
-    R c = rdiv(a * fb - b * fa, fb - fa);
+    R c = rdiv<R, EOS>(a * fb - b * fa, fb - fa);
     if (!(c2p_above(c, a) && c2p_above(b, c))) c = R(0.5) * (a + b);
     if (!(c2p_above(c, a) && c2p_above(b, c))) {
       *root = c; *hi_out = b; *iters = it;
@@ -1100,10 +1100,10 @@ __device__ __forceinline__ bool c2p_presolve32(const KParams& P, const C2PInv<do
   const float top = EOS ? P.top_f : 1.f, h0sq = EOS ? P.h0sq_f : 1.f;
   float mup = top, root, hiv;
   int it;
-  const float f1 = c2p_aux<float>(I, h0sq, top);
+  const float f1 = c2p_aux<float, EOS>(I, h0sq, top);
   if (f1 > 0.f) {
-    auto fa = [&](float mu) { return c2p_aux<float>(I, h0sq, mu); };
-    if (illinois<float>(fa, 0.f, top, -1.f, f1, 1e-3f, 40, &root, &hiv, &it) == 0) mup = hiv;
+    auto fa = [&](float mu) { return c2p_aux<float, EOS>(I, h0sq, mu); };
+    if (illinois<float, EOS>(fa, 0.f, top, -1.f, f1, 1e-3f, 40, &root, &hiv, &it) == 0) mup = hiv;
   }
   C2PVal<float> E;
   int kh = -1;   // temperature interval of the last evaluation (table)
@@ -1122,7 +1122,7 @@ __device__ __forceinline__ bool c2p_presolve32(const KParams& P, const C2PInv<do
       if (!(fa < 0.f) || !(fb >= 0.f)) return false;
       phase = 3;
     } else {
-      if (fc == 0.f) { *islope = fdiv(b - a, gb - ga); a = mu; b = mu; break; }
+      if (fc == 0.f) { *islope = rdiv<float, EOS>(b - a, gb - ga); a = mu; b = mu; break; }
       if (fc < 0.f) {
         a = mu; fa = ga = fc;
         if (side == -1) fb *= 0.5f;
@@ -1135,14 +1135,14 @@ __device__ __forceinline__ bool c2p_presolve32(const KParams& P, const C2PInv<do
       ++k;
     }
     if (k >= 12 || !(b - a > 1e-4f * b)) break;
-    mu = fdiv(a * fb - b * fa, fb - fa);
+    mu = rdiv<float, EOS>(a * fb - b * fa, fb - fa);
     if (!(mu > a && mu < b)) mu = 0.5f * (a + b);
     if (!(mu > a && mu < b)) break;
   }
   *lo = a;
   *hi = b;
   *khint = kh;
-  if (b > a) *islope = fdiv(b - a, gb - ga);
+  if (b > a) *islope = rdiv<float, EOS>(b - a, gb - ga);
   float c = a - ga * *islope;
   if (!(c > a && c < b)) c = 0.5f * (a + b);
   *est = c;
@@ -1317,20 +1317,20 @@ __device__ __forceinline__ int con2prim_cell(const Site& site, const KParams& P,
         If.ye = 0.f;
         if (isfinite(If.r2) && isfinite(If.b2) && isfinite(If.rb * If.rb)) {
           const float topf = EOS ? P.top_f : 1.f, h0sqf = EOS ? P.h0sq_f : 1.f;
-          const float f1 = c2p_aux<float>(If, h0sqf, topf);
+          const float f1 = c2p_aux<float, EOS>(If, h0sqf, topf);
           float rootf, hif;
           if (f1 > 0.f) {
-            auto fa = [&](float mu) { return c2p_aux<float>(If, h0sqf, mu); };
-            if (illinois<float>(fa, 0.f, topf, -1.f, f1, 1e-3f, P.max_iter, &rootf, &hif, &it_aux) == 0)
+            auto fa = [&](float mu) { return c2p_aux<float, EOS>(If, h0sqf, mu); };
+            if (illinois<float, EOS>(fa, 0.f, topf, -1.f, f1, 1e-3f, P.max_iter, &rootf, &hif, &it_aux) == 0)
               mup = fmin(f2d_exact(hif), top);
           }
           return mup;
         }
       }
-      const double f1 = c2p_aux<double>(I, h0sq, top);
+      const double f1 = c2p_aux<double, EOS>(I, h0sq, top);
       if (f1 > 0.0) {
-        auto fa = [&](double mu) { return c2p_aux<double>(I, h0sq, mu); };
-        if (illinois<double>(fa, 0.0, top, -1.0, f1, 1e-3, P.max_iter, &rt, &hi, &it_aux) == 0) mup = hi;
+        auto fa = [&](double mu) { return c2p_aux<double, EOS>(I, h0sq, mu); };
+        if (illinois<double, EOS>(fa, 0.0, top, -1.0, f1, 1e-3, P.max_iter, &rt, &hi, &it_aux) == 0) mup = hi;
       }
       return mup;
     };
