@@ -957,10 +957,10 @@ def main():
         stv = str_.to(torch.int32)
         rk = {"ms_per_rk3_step": ms_rk, "stages": 3, "cfl": 0.25, "dt": G.gr_driver_dt(drv),
               "cell_updates_per_s_per_stage": 3 * cells * world / (ms_rk / 1e3),
-              "launches_per_step": 1 + 1 + 1 + 3 * 6 + 2 * 1,
+              "launches_per_step": 1 + 1 + 1 + 3 * 7 + 2 * 1,
               "ghost_fill": {"ms": ms_gf, "bytes": gb, "GB_per_s": gb / (ms_gf / 1e3) / 1e9},
               "failed_cells_after": int(((stv & 2) != 0).sum().item()),
-              "note": "graph of ghost fill (1 kernel) + grid dt (1) + the FP32 conversion of W and B (1) + 3 x (6 stage "
+              "note": "graph of ghost fill (1 kernel) + grid dt (1) + the FP32 conversion of W and B (1) + 3 x (7 stage "
                       "kernels) + 2 inter-stage ghost fills (FP64 and FP32 copies together); the later stages read "
                       "the FP32 copies their predecessors wrote; static metric given with its FP32 copy; outflow "
                       "boundaries; the state evolves over warm-up and timed steps"}
@@ -1153,7 +1153,7 @@ def main():
 
     # cell prep, faces, edges, CT, update, con2prim (+ the FP32 cast on the mixed path) per stage
     # cell prep, faces, edges, CT, update, con2prim per stage (the steady-state mixed stage converts nothing)
-    launches = a.steps * 6
+    launches = a.steps * 7   # cell prep, faces, edges, CT, update, jobs, con2prim
     fp64 = None
     if "fp64" in results and head != "fp64":
         fp64 = {"value": cells * world / (results["fp64"]["ms"] / 1e3), "ms_per_step": results["fp64"]["ms"],

@@ -15,8 +15,8 @@
 //   k_update     FP64 path: flux divergence + geometric sources (Eq. claw, Eq. hydsrc_def)
 //                accumulated in FP64 and the atmosphere test (Sec. 3.5); mixed path: D' and the
 //                atmosphere test only; atmosphere cells are reset, the others queued for k_c2p
-//   k_c2p        on the compacted job list: (mixed path) the cell's U' as above, then FP64 con2prim
-//                (Sec. 3.5, App. A)
+//   k_jobs       mixed path: the U' of the queued cells, as above
+//   k_c2p        on the compacted job list: FP64 con2prim (Sec. 3.5, App. A) of U'
 //
 // Kernels that evaluate the EOS are instantiated per EOS (ideal gas / table) as well as per R.
 // Every kernel but the sweep and k_c2p takes one work item (block, direction, first element) per CTA;
