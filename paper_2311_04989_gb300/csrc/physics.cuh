@@ -245,7 +245,8 @@ __device__ __forceinline__ void cell_metric4_dv(const DBlock& b, const InView<fl
 // Cell-centre value of components [c0, nc) and, if dv != nullptr, derivatives d_k of components
 // [0, 10) (alpha, beta, gamma), computed in R from the FP64 vertex pools.  The derivative along k is
 // written as vertex differences so that it vanishes exactly on a constant field.
-template <class R>
+// FIX (FP64): in fixed point; without it by FP64 additions, for the forms of con2prim that keep their roundings.
+template <class R, bool FIX = true>
 __device__ __forceinline__ void cell_metric(const DBlock& b, const InView<R>& m, int order, int i,
                                             int j, int k, int c0, int nc, R* val, R (*dv)[10]) {
   const long long base = b.vert;
@@ -260,7 +261,7 @@ __device__ __forceinline__ void cell_metric(const DBlock& b, const InView<R>& m,
       R f[8];
 #pragma unroll
       for (int t = 0; t < 8; ++t) f[t] = a[v[t]];
-      if constexpr (sizeof(R) == sizeof(double)) {   // in fixed point (FP64 pipe: 32 additions a component)
+      if constexpr (FIX && sizeof(R) == sizeof(double)) {   // in fixed point (FP64 pipe: 32 additions a component)
         if (dv && c < 10) {
           haar8_64(f, &val[c], &dv[0][c], &dv[1][c], &dv[2][c]);
           dv[0][c] *= ix;
@@ -291,7 +292,7 @@ __device__ __forceinline__ void cell_metric(const DBlock& b, const InView<R>& m,
 #pragma unroll
     for (int c = c0; c < nc; ++c) {
       const R* a = m.M[c];
-      if constexpr (sizeof(R) == sizeof(double)) {
+      if constexpr (FIX && sizeof(R) == sizeof(double)) {
         if (!dv || c >= 10) {   // no derivatives: by planes in fixed point
           val[c] = lagr_cell64(b, a, base, i, j, k);
           continue;
@@ -848,10 +849,12 @@ struct C2PMet {
 // Forms of con2prim_cell.  PLAIN: the FP64 path and gr_con2prim, step for step the oracle's.  NEWTON: the mixed
 // stage (Newton steps from the FP32 pre-solve's root, whether or not its bracket was asked for).  BRACKET: the
 // mixed stage with a learned bracket, and the stages of an RK driver step without the pre-solve (FP32 bracket top,
-// two-division master function).  BRACKET keeps its roundings (order-2 metric) whatever is done to the speed: its last iterate can
+// two-division master function).  BRACKET keeps its roundings whatever is done to the speed: its last iterate can
 // sit anywhere in the final bracket (1e-10 wide), set by f's rounding noise, and the next stage of the step rounds
 // the primitives to FP32, so a better root turns some of those over (p by up to 3e-7 after the step); one stage
-// moves by less than 1e-10.
+// moves by less than 1e-10.  PLAIN keeps those of its metric too: gr_con2prim
+// called again on its own output meets cells that a limit left exactly on it, and one rounding of sqrt(gamma) decides
+// whether their status shows the limit again.
 enum { C2P_PLAIN = 0, C2P_BRACKET = 1, C2P_NEWTON = 2 };
 
 // mixed forms: sqrt(gamma) and its inverse from one reciprocal square root, sg = det rsqrt(det), in place of

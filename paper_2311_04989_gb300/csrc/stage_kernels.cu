@@ -354,16 +354,10 @@ template <int MODE = C2P_PLAIN>
 __device__ __forceinline__ void cell_gamma64(const DBlock& b, const InView<double>& m, int i, int j, int k,
                                              C2PMet& M) {
   double val[10];
-  if (MODE == C2P_BRACKET && m.order == 2) {   // that form keeps its roundings (physics.cuh)
-    const long long v0 = b.vert + vix(b, i, j, k);
-    const int sy = b.N[0] + 1, sz = sy * (b.N[1] + 1);
-#pragma unroll
-    for (int c = 4; c < 10; ++c) {
-      const double* a = m.M[c] + v0;
-      val[c] = 0.125 * (((a[0] + a[1]) + (a[sy] + a[sy + 1])) + ((a[sz] + a[sz + 1]) + (a[sz + sy] + a[sz + sy + 1])));
-    }
-  } else if (MODE == C2P_BRACKET || m.order == 2) {
-    cell_metric<double>(b, m, MODE == C2P_BRACKET ? m.order : 2, i, j, k, 4, 10, val, nullptr);
+  if constexpr (MODE != C2P_NEWTON) {   // those forms keep their roundings (physics.cuh)
+    cell_metric<double, false>(b, m, m.order, i, j, k, 4, 10, val, nullptr);
+  } else if (m.order == 2) {
+    cell_metric<double>(b, m, 2, i, j, k, 4, 10, val, nullptr);
   } else {   // one copy of the long interpolation, its results through local memory
     double g4[6];
 #pragma unroll 1
@@ -472,9 +466,10 @@ __device__ __forceinline__ bool update_cell(const Work& w, const DBlock& b, cons
   }
 }
 
-// FP32: at most 64 registers (four 256-thread CTAs per SM): the mixed update is bound by load latency
+// FP32: at most 64 registers (four 256-thread CTAs per SM): the mixed update is bound by load latency.  FP64: 128 (48
+// AMR-like blocks: 0.72 ms at the 212 it would take, 0.62 at 128, 0.62 at 96, 0.63 at 168): FP64 pipe and latency
 template <class R, int EOS>
-__global__ void __launch_bounds__(kMaxTile, sizeof(R) == sizeof(float) ? 4 : 0) k_update(const DBlock* __restrict__ blocks, const Work* __restrict__ work,
+__global__ void __maxnreg__(sizeof(R) == sizeof(float) ? 64 : 128) k_update(const DBlock* __restrict__ blocks, const Work* __restrict__ work,
                                                      int nwork, const __grid_constant__ InView<R> in,
                                                      const __grid_constant__ StateView s,
                                                      const __grid_constant__ Workspace ws,
@@ -560,7 +555,8 @@ struct PoolSite {
 // Bound by the FP64 pipe (75-84 % busy).  On the AMR-like batch (256 blocks, FP32 pre-solve) the FP64
 // instructions per warp went from 640 to about 230 and the time with k_jobs from 5.09 to 2.5 ms: divisions and
 // roots as integers (soft64.cuh), one evaluation site per solve, Newton steps, the cell metric by fixed-point
-// means.  gr_con2prim on 64 x 32^3 cells 4.79 -> 2.84 ms (ideal gas), on 32 x 32^3 with the table 7.4 -> 4.5 ms.
+// means.  Registers: NEWTON 96 (80 2.44 ms, 112 2.40, 128 2.36 with k_jobs, but a 64^3 star then 178 us for 168),
+// BRACKET and PLAIN 128 (RK3 step of 512 blocks 10.8 ms; 112 11.9, 96 12.0, 168 10.9).  gr_con2prim on 64 x 32^3 cells 4.79 -> 2.84 ms (ideal gas), on 32 x 32^3 with the table 7.4 -> 4.5 ms.
 template <int EOS, int MODE>
 __global__ void __maxnreg__(MODE == C2P_NEWTON ? 96 : 128) k_c2p(const DBlock* __restrict__ blocks, const __grid_constant__ InView<double> in64,
                                        const __grid_constant__ StateView s, const __grid_constant__ Workspace ws,
