@@ -556,7 +556,8 @@ struct PoolSite {
 // instructions per warp went from 640 to about 230 and the time with k_jobs from 5.09 to 2.5 ms: divisions and
 // roots as integers (soft64.cuh), one evaluation site per solve, Newton steps, the cell metric by fixed-point
 // means.  Registers: NEWTON 96 (80 2.44 ms, 112 2.40, 128 2.36 with k_jobs, but a 64^3 star then 178 us for 168),
-// BRACKET and PLAIN 128 (RK3 step of 512 blocks 10.8 ms; 112 11.9, 96 12.0, 168 10.9).  gr_con2prim on 64 x 32^3 cells 4.80 -> 2.47 ms (ideal gas), on 32 x 32^3 with the table 7.4 -> 4.5 ms.
+// BRACKET and PLAIN 128 (RK3 step of 512 blocks 10.8 ms; 112 11.9, 96 12.0, 168 10.9).  gr_con2prim
+// on 64 x 32^3 cells 4.80 -> 2.47 ms (ideal gas), on 32 x 32^3 with the table 7.4 -> 4.5 ms.
 template <int EOS, int MODE>
 __global__ void __maxnreg__(MODE == C2P_NEWTON ? 96 : 128) k_c2p(const DBlock* __restrict__ blocks, const __grid_constant__ InView<double> in64,
                                        const __grid_constant__ StateView s, const __grid_constant__ Workspace ws,
