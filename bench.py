@@ -339,7 +339,7 @@ def run_reference(a):
 # ---------------------------------------------------------------------------------------------
 # the sources the stage kernels are compiled from (a change to any of them invalidates the
 # committed DRAM traffic; the driver, matter-source and level-boundary kernels do not enter)
-STAGE_SOURCES = ("eos.cuh", "faces_core.cuh", "faces_f32.cu", "faces_f64.cu", "faces_impl.cuh", "internal.h", "mlp.cuh",
+STAGE_SOURCES = ("castlist.h", "eos.cuh", "faces_core.cuh", "faces_f32.cu", "faces_f64.cu", "faces_impl.cuh", "internal.h", "mlp.cuh",
                  "physics.cuh", "soft64.cuh", "stage_common.cuh", "stage_kernels.cu", "update_common.cuh")
 
 

@@ -27,22 +27,15 @@
 
 #include "internal.h"
 #include "physics.cuh"
+#include "castlist.h"
 #include "stage_common.cuh"
 #include "update_common.cuh"
-
 
 namespace grs {
 
 // ------------------------------------------------------------------------------------------------
-// k_cast: FP64 -> FP32 copies of up to 24 pools
+// k_cast: FP64 -> FP32 copies of the pools of a CastList
 // ------------------------------------------------------------------------------------------------
-struct CastList {
-  const double* src[24];
-  float* dst[24];
-  long long n[24];
-  int count;
-};
-
 __global__ void __launch_bounds__(256) k_cast(const __grid_constant__ CastList L) {
   stage_begin();
   const int seg = blockIdx.y;
@@ -809,36 +802,24 @@ static InView<float> view32(const MetricView& m, const StateView& s, const Shado
   return v;
 }
 
-// the conversions a mixed stage needs: W and B unless the caller gave copies, the metric unless the
-// caller gave one or (cast_metric = false) the previous stage on this mesh made it
+// the conversions of a mixed stage (stage_casts), in one launch
 static cudaError_t launch_cast(const MetricView& m, const StateView& s, const Shadow& sh, int eos,
                                cudaStream_t st, bool cast_metric) {
   CastList L;
-  int k = 0;
-  const int nw = eos == GR_EOS_TABLE ? 6 : 5;   // rho, u~^i, p[, Y_e]
-  if (!s.W32[0]) {
-    for (int q = 0; q < nw; ++q) { L.src[k] = s.W[q]; L.dst[k] = sh.W[q]; L.n[k] = sh.ncell; ++k; }
-    for (int d = 0; d < 3; ++d) { L.src[k] = s.B[d]; L.dst[k] = sh.B[d]; L.n[k] = sh.nface[d]; ++k; }
-  }
-  const int ncomp = (cast_metric && !m.v32[0]) ? (m.k_zero ? 10 : 16) : 0;
-  for (int c = 0; c < ncomp; ++c) { L.src[k] = m.v[c]; L.dst[k] = sh.M[c]; L.n[k] = sh.nvert; ++k; }
-  L.count = k;
-  if (k == 0) return cudaSuccess;
+  if (!stage_casts(m, s, sh, eos, cast_metric, L)) return cudaErrorInvalidValue;
+  if (L.count == 0) return cudaSuccess;
   // two 256-thread CTAs per SM and pool, striding over it
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1) nsm = 1;
-  dim3 grid(2 * nsm, k);
+  dim3 grid(2 * nsm, L.count);
   k_cast<<<grid, 256, 0, st>>>(L);
   return cudaGetLastError();
 }
 
 cudaError_t launch_cast_pool(const double* src, float* dst, long long n, cudaStream_t st) {
   CastList L{};
-  L.src[0] = src;
-  L.dst[0] = dst;
-  L.n[0] = n;
-  L.count = 1;
+  L.add(src, dst, n);
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1) nsm = 1;
