@@ -69,8 +69,9 @@ enum { GR_EOS_IDEAL = 0, GR_EOS_TABLE = 1 };            /* Sec. 2.2.1 */
  * none, an FP32 pre-solve (the bracket narrowed in FP32 to 1e-4 of its upper end, then widened by 4e-6),
  * the learned bracket of a small network (gr_mlp_*), or GR_GUESS_AUTO: the mesh's choice between none and
  * the FP32 pre-solve for the call's precision and EOS, made by gr_autotune by timing the stage with each
- * (none until the mesh is tuned; gr_mesh_get_guess reads it).  The mixed gr_stage starts its FP64 iteration from an
- * FP32 solve with either of none and FP32; they differ in the status bit of a rejected proposal there. */
+ * (none until the mesh is tuned; gr_mesh_get_guess reads it).  A mixed stage with the
+ * FP32 pre-solve takes Newton steps in FP64 from its root, one without it the bracketed solve; the stages of
+ * gr_driver_step take what gr_stage takes. */
 enum { GR_GUESS_NONE = 0, GR_GUESS_FP32 = 1, GR_GUESS_MLP = 2, GR_GUESS_AUTO = 3 };
 
 /* Atmosphere band (gr_params.atm_band) for the mixed path: its atmosphere test compares D' with the

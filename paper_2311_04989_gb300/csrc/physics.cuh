@@ -846,15 +846,15 @@ struct C2PMet {
   double isg;   // 1/sqrt(gamma), formed only by the mixed forms
 };
 
-// Forms of con2prim_cell.  PLAIN: the FP64 path and gr_con2prim, step for step the oracle's.  NEWTON: the mixed
-// stage (Newton steps from the FP32 pre-solve's root, whether or not its bracket was asked for).  BRACKET: the
-// mixed stage with a learned bracket, and the stages of an RK driver step without the pre-solve (FP32 bracket top,
-// two-division master function).  BRACKET keeps its roundings whatever is done to the speed: its last iterate can
-// sit anywhere in the final bracket (1e-10 wide), set by f's rounding noise, and the next stage of the step rounds
-// the primitives to FP32, so a better root turns some of those over (p by up to 3e-7 after the step); one stage
-// moves by less than 1e-10.  PLAIN keeps those of its metric too: gr_con2prim
-// called again on its own output meets cells that a limit left exactly on it, and one rounding of sqrt(gamma) decides
-// whether their status shows the limit again.
+// Forms of con2prim_cell, chosen by the call's precision and bracket proposal alone.  PLAIN: the FP64 path and
+// gr_con2prim, step for step the oracle's.  NEWTON: the mixed stage with the FP32 pre-solve (Newton steps from its
+// root).  BRACKET: the mixed stage without a proposal or with a learned one (FP32 bracket top, two-division master
+// function).  BRACKET keeps its roundings whatever is done to the speed: its last iterate can sit anywhere in the
+// final bracket (1e-10 wide), set by f's rounding noise, and the next stage of an RK step rounds the primitives to FP32, so
+// a better root turns some of those over (p of an RK3 step of 512 blocks by up to 1e-7 with NEWTON in its place, though
+// the step then takes 6.7 ms for 11.0 and its error against 64 bits stays 2.0e-7).  PLAIN keeps those of its metric too:
+// gr_con2prim called again on its own output meets cells that a limit left exactly on it, and one rounding of sqrt(gamma)
+// decides whether their status shows the limit again.
 enum { C2P_PLAIN = 0, C2P_BRACKET = 1, C2P_NEWTON = 2 };
 
 // mixed forms: sqrt(gamma) and its inverse from one reciprocal square root, sg = det rsqrt(det), in place of
@@ -1376,7 +1376,7 @@ __device__ __forceinline__ int con2prim_cell(const Site& site, const KParams& P,
           root = mu;
           fresh = true;
           // the proposed bracket would have shown no sign change
-          if (P.c2p_guess == GR_GUESS_FP32 && (gtp64(f2d_exact(lo32) * (1.0 - 4e-6), mu) || gtp64(mu, f2d_exact(hi32) * (1.0 + 4e-6))))
+          if (gtp64(f2d_exact(lo32) * (1.0 - 4e-6), mu) || gtp64(mu, f2d_exact(hi32) * (1.0 + 4e-6)))
             st |= GR_ST_GUESS_REJECTED;
         }
       }

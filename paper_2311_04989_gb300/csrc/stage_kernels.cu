@@ -837,8 +837,7 @@ template <int EOS, bool MIXED>
 static void launch_c2p(const DBlock* blocks, const KLaunch& q, const InView<double>& in64, const StateView& s,
                        const Workspace& ws, const KParams& kp, cudaStream_t st, bool overlap) {
   if constexpr (!MIXED) launch_c2p_m<EOS, C2P_PLAIN>(blocks, q, in64, s, ws, kp, st, overlap);
-  else if (kp.c2p_guess == GR_GUESS_FP32 || (kp.c2p_guess == GR_GUESS_NONE && !kp.dt_dev))
-    launch_c2p_m<EOS, C2P_NEWTON>(blocks, q, in64, s, ws, kp, st, overlap);
+  else if (kp.c2p_guess == GR_GUESS_FP32) launch_c2p_m<EOS, C2P_NEWTON>(blocks, q, in64, s, ws, kp, st, overlap);
   else launch_c2p_m<EOS, C2P_BRACKET>(blocks, q, in64, s, ws, kp, st, overlap);
 }
 
