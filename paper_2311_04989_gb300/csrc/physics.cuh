@@ -245,7 +245,9 @@ __device__ __forceinline__ void cell_metric4_dv(const DBlock& b, const InView<fl
 // Cell-centre value of components [c0, nc) and, if dv != nullptr, derivatives d_k of components
 // [0, 10) (alpha, beta, gamma), computed in R from the FP64 vertex pools.  The derivative along k is
 // written as vertex differences so that it vanishes exactly on a constant field.
-// FIX (FP64): in fixed point; without it by FP64 additions, for the forms of con2prim that keep their roundings.
+// FIX (FP64): in fixed point; without it by FP64 additions, for gamma_ij where an atmosphere test or a reset depends on
+// sqrt(gamma): con2prim (but for its NEWTON form), prim2con and, here too, the update with its derivatives, so that all
+// of them decide on the same bits and leave the same D = sqrt(gamma) rho_atm.
 template <class R, bool FIX = true>
 __device__ __forceinline__ void cell_metric(const DBlock& b, const InView<R>& m, int order, int i,
                                             int j, int k, int c0, int nc, R* val, R (*dv)[10]) {
@@ -264,6 +266,7 @@ __device__ __forceinline__ void cell_metric(const DBlock& b, const InView<R>& m,
       if constexpr (FIX && sizeof(R) == sizeof(double)) {   // in fixed point (FP64 pipe: 32 additions a component)
         if (dv && c < 10) {
           haar8_64(f, &val[c], &dv[0][c], &dv[1][c], &dv[2][c]);
+          if (c >= 4) val[c] = scale64<3>(((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])));
           dv[0][c] *= ix;
           dv[1][c] *= iy;
           dv[2][c] *= iz;

@@ -600,7 +600,8 @@ __global__ void __launch_bounds__(kTile) k_prim2con(const DBlock* __restrict__ b
   int p[3];
   if (!decode<R_INTERIOR, 0>(w, b, p)) return;
   double val[16];
-  cell_metric<double>(b, m, m.order, p[0], p[1], p[2], 0, 10, val, nullptr);
+  cell_metric<double>(b, m, m.order, p[0], p[1], p[2], 0, 4, val, nullptr);
+  cell_metric<double, false>(b, m, m.order, p[0], p[1], p[2], 4, 10, val, nullptr);   // con2prim's sqrt(gamma)
   CellMet<double> M;
   cellmet_from<double>(val, true, M);
   const long long c = b.cell + cix(b, p[0], p[1], p[2]);
