@@ -77,7 +77,7 @@ __device__ __forceinline__ void face_flux(const R* L, const R* Rr, const R met[1
   wr[5] = EOS ? Rr[NV - 1] : R(0);
   const R det = det3(met + 4);
   const R sg = sqrt_r(det);
-  const R gdd = inv_dd<R, EOS>(met + 4, D, det);
+  const R gdd = inv_dd(met + 4, D, det);
   R BL[3], BR[3];
   BL[D] = Bn; BR[D] = Bn;
   BL[t1] = L[5] * sg; BL[t2] = L[6] * sg;
@@ -85,7 +85,7 @@ __device__ __forceinline__ void face_flux(const R* L, const R* Rr, const R met[1
   R UL[7], FL[7], UR[7], FR[7], lmL, lpL, lmR, lpR;
   face_state<R, EOS>(D, met, sg, gdd, kp, wl, BL, UL, FL, &lmL, &lpL);
   face_state<R, EOS>(D, met, sg, gdd, kp, wr, BR, UR, FR, &lmR, &lpR);
-  hlle<R, EOS>(UL, UR, FL, FR, lmL, lpL, lmR, lpR, F);
+  hlle<R>(UL, UR, FL, FR, lmL, lpL, lmR, lpR, F);
   if constexpr (EOS == GR_EOS_TABLE) *ye_up = F[0] > R(0) ? wl[5] : wr[5];
   else *ye_up = R(0);
 }

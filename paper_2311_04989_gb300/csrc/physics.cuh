@@ -18,11 +18,18 @@ namespace grs {
 // small helpers
 // ------------------------------------------------------------------------------------------------
 // square root in precision R: the IEEE square root in FP64; in FP32 (the mixed path) the hardware's
-// approximate square root (PTX sqrt.approx.ftz.f32, relative error of the order of one FP32 ulp, subnormals as
-// zero), one or two instructions instead of the correctly rounded sequence
+// approximate square root (PTX sqrt.approx.f32, relative error of the order of one FP32 ulp), a few
+// instructions instead of the correctly rounded sequence
 template <class R> __device__ __forceinline__ R sqrt_r(R x);
 template <> __device__ __forceinline__ double sqrt_r(double x) { return sqrt64(x); }
 template <> __device__ __forceinline__ float sqrt_r(float x) {
+  float y;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+// the same for an x that is zero or not subnormal: sqrt_r without its scaling of subnormal operands, the same bits
+template <class R> __device__ __forceinline__ R sqrt_n(R x) { return sqrt_r(x); }
+template <> __device__ __forceinline__ float sqrt_n(float x) {
   float y;
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
@@ -33,22 +40,24 @@ template <> __device__ __forceinline__ float sqrt_r(float x) {
 template <class R> __device__ __forceinline__ R sqrt_w(R x) { return sqrt64(x); }
 template <> __device__ __forceinline__ float sqrt_w(float x) { return sqrtf(x); }
 
-// a/b in FP32 as a times the hardware reciprocal of b, with subnormal operands and results flushed to zero: the
-// bits of __fdividef for normal ones, without its scaling of the others (four to five instructions for two; a
-// face takes some seventy divisions)
-__device__ __forceinline__ float fdiv(float a, float b) {
+// a/b: IEEE division in FP64; the fast approximate FP32 division (2 ulp) on the mixed path
+template <class R> __device__ __forceinline__ R rdiv(R a, R b);
+template <> __device__ __forceinline__ double rdiv(double a, double b) { return div64(a, b); }
+template <> __device__ __forceinline__ float rdiv(float a, float b) { return __fdividef(a, b); }
+// __fdividef for a divisor that is not subnormal: a times the hardware reciprocal of b without the scaling of subnormal
+// divisors, the same bits otherwise, subnormal dividends and quotients included (two instructions for four to five;
+// a face takes some fifty of them)
+__device__ __forceinline__ float fdiv_n(float a, float b) {
   float y;
-  asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
-  return y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(b));
+  return __fmul_rn(a, y);
 }
-// a/b: IEEE division in FP64; the fast approximate FP32 division (2 ulp) on the mixed path, fdiv but with a table:
-// there it changes which products the compiler fuses, the FP32 fluxes by their rounding, and the pre-solve's bracket
-// (and with it the status bit of a rejected one)
+// rdiv for such a divisor.  With a table it is rdiv: there another division changes which products the compiler fuses,
+// the FP32 fluxes by their rounding, and the pre-solve's bracket (and with it the status bit of a rejected one)
 template <class R, int EOS = GR_EOS_IDEAL>
-__device__ __forceinline__ R rdiv(R a, R b) {
-  if constexpr (sizeof(R) == sizeof(double)) return div64(a, b);
-  else if constexpr (EOS == GR_EOS_TABLE) return __fdividef(a, b);
-  else return fdiv(a, b);
+__device__ __forceinline__ R rdiv_n(R a, R b) {
+  if constexpr (sizeof(R) == sizeof(float) && EOS == GR_EOS_IDEAL) return fdiv_n(a, b);
+  else return rdiv(a, b);
 }
 
 // x 2^-K
@@ -94,13 +103,13 @@ __device__ __forceinline__ R det3(const R g[6]) {
 }
 
 // gamma^{dd} = cofactor_dd / det
-template <class R, int EOS = GR_EOS_IDEAL>
+template <class R>
 __device__ __forceinline__ R inv_dd(const R g[6], int d, R det) {
   R c;
   if (d == 0) c = g[3] * g[5] - g[4] * g[4];
   else if (d == 1) c = g[0] * g[5] - g[2] * g[2];
   else c = g[0] * g[3] - g[1] * g[1];
-  return rdiv<R, EOS>(c, det);
+  return rdiv(c, det);
 }
 
 // full inverse
@@ -393,10 +402,10 @@ __device__ __forceinline__ float weno5(float v0, float v1, float v2, float v3, f
   float q[3], bk[3];
   wenoz_parts(v0, v1, v2, v3, v4, q, bk);
   const float e = 1e-18f;
-  const float w0 = fdiv(0.1f, xm(xa(bk[0], e), xa(bk[0], e)));
-  const float w1 = fdiv(0.6f, xm(xa(bk[1], e), xa(bk[1], e)));
-  const float w2 = fdiv(0.3f, xm(xa(bk[2], e), xa(bk[2], e)));
-  return fdiv(xa(xa(xm(w0, q[0]), xm(w1, q[1])), xm(w2, q[2])), xa(xa(w0, w1), w2));
+  const float w0 = __fdividef(0.1f, xm(xa(bk[0], e), xa(bk[0], e)));
+  const float w1 = __fdividef(0.6f, xm(xa(bk[1], e), xa(bk[1], e)));
+  const float w2 = __fdividef(0.3f, xm(xa(bk[2], e), xa(bk[2], e)));
+  return __fdividef(xa(xa(xm(w0, q[0]), xm(w1, q[1])), xm(w2, q[2])), xa(xa(w0, w1), w2));
 }
 
 // PPM: fourth-order interface values limited by the extremum-preserving criterion of Colella & Sekora,
@@ -452,10 +461,11 @@ __device__ __forceinline__ void ppm_cell(R v0, R v1, R v2, R v3, R v4, R* qm, R*
 // WENOZ of both face states at once in FP32 (packed FP32x2 arithmetic: one instruction per operation
 // for both).  Lane x: the L state, wenoz of cells f-3 .. f+1; lane y: the R state, wenoz of the mirror
 // image f+2 .. f-2.  Both lanes take the same operations, so a mirror-symmetric stencil still gives
-// L == R bitwise.  Weights d_k (1 + tau5/(beta_k + eps)) from the fast reciprocal of beta_k + eps.
+// L == R bitwise.  Weights d_k (1 + tau5/(beta_k + eps)) from the fast reciprocal of beta_k + eps (1e-30 or
+// more; the divisor of the sum is 1 or more).
 __device__ __forceinline__ float2 pk(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ float2 pk1(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 prcp(float2 a) { return make_float2(fdiv(1.f, a.x), fdiv(1.f, a.y)); }
+__device__ __forceinline__ float2 prcp(float2 a) { return make_float2(fdiv_n(1.f, a.x), fdiv_n(1.f, a.y)); }
 
 __device__ __forceinline__ void wenoz_pair(const float s[6], float eps, float* L, float* Rr) {
   const float2 v0 = pk(s[0], s[5]), v1 = pk(s[1], s[4]), v2 = pk(s[2], s[3]);
@@ -487,8 +497,8 @@ __device__ __forceinline__ void wenoz_pair(const float s[6], float eps, float* L
   const float2 w2 = __ffma2_rn(pk1(0.3f), r2, pk1(0.3f));
   const float2 num = __ffma2_rn(w2, q2, __ffma2_rn(w1, q1, __fmul2_rn(w0, q0)));
   const float2 den = __fadd2_rn(__fadd2_rn(w0, w1), w2);
-  *L = fdiv(num.x, den.x);
-  *Rr = fdiv(num.y, den.y);
+  *L = fdiv_n(num.x, den.x);
+  *Rr = fdiv_n(num.y, den.y);
 }
 
 // WENOZ and WENO5 of both face states in FP64, in the differences d_i = s_{i+1} - s_i of the stencil, which the
@@ -603,8 +613,8 @@ __device__ __forceinline__ void eos_rhoh_cs2(const KParams& kp, R rho, R p, R ye
     R gam;
     if constexpr (sizeof(R) == sizeof(float)) gam = kp.gamma_f;
     else gam = kp.gamma_ad;
-    *rhoh = rho + gam * rdiv<R, EOS>(p, gam - R(1));
-    *cs2 = rdiv<R, EOS>(gam * p, *rhoh);
+    *rhoh = rho + gam * rdiv(p, gam - R(1));
+    *cs2 = rdiv(gam * p, *rhoh);
   } else {
     tab_thermo_p<R>(tab_of<R>(kp), rho, p, ye, rhoh, cs2, (R*)nullptr);
   }
@@ -627,9 +637,9 @@ __device__ __forceinline__ void face_state(int d, const R met[10], R sg, R gdd, 
   R utl[3];
   lower3(g, ut, utl);
   const R W = sqrt_w(R(1) + ut[0] * utl[0] + ut[1] * utl[1] + ut[2] * utl[2]);
-  const R iW = rdiv<R, EOS>(R(1), W);
-  const R ia = rdiv<R, EOS>(R(1), alpha);
-  const R isg = rdiv<R, EOS>(R(1), sg);
+  const R iW = rdiv_n<R, EOS>(R(1), W);   // W >= 1
+  const R ia = rdiv(R(1), alpha);
+  const R isg = rdiv(R(1), sg);
   R v[3], vl[3], vt[3], Bu[3], Bl[3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
@@ -670,20 +680,20 @@ __device__ __forceinline__ void face_state(int d, const R met[10], R sg, R gdd, 
   F[5] = alpha * (Bd[t1] * vt[d] - Bd[d] * vt[t1]);
   F[6] = alpha * (Bd[t2] * vt[d] - Bd[d] * vt[t2]);
   // fast speeds
-  const R ca2 = rdiv<R, EOS>(b2, e);
+  const R ca2 = rdiv(b2, e);
   const R c2 = cs2 + ca2 - cs2 * ca2;
   const R v2 = v[0] * vl[0] + v[1] * vl[1] + v[2] * vl[2];
   R disc = (R(1) - v2) * (gdd * (R(1) - v2 * c2) - v[d] * v[d] * (R(1) - c2));
   disc = rpos(disc) ? disc : R(0);
   const R cr = sqrt_r(c2) * sqrt_r(disc);
-  const R iden = rdiv<R, EOS>(R(1), R(1) - v2 * c2);
+  const R iden = rdiv_n<R, EOS>(R(1), R(1) - v2 * c2);   // 0, or an ulp of 1 or more
   const R vc = v[d] * (R(1) - c2);
   *lp = alpha * (vc + cr) * iden - beta[d];
   *lm = alpha * (vc - cr) * iden - beta[d];
 }
 
 // HLLE (lam+ = max(0, ...), lam- = min(0, ...); equal speeds give the mean flux)
-template <class R, int EOS = GR_EOS_IDEAL>
+template <class R>
 __device__ __forceinline__ void hlle(const R UL[7], const R UR[7], const R FL[7], const R FR[7], R lmL,
                                      R lpL, R lmR, R lpR, R out[7]) {
   const R lp = rmax(R(0), rmax(lpL, lpR));
@@ -694,7 +704,7 @@ __device__ __forceinline__ void hlle(const R UL[7], const R UR[7], const R FL[7]
     for (int v = 0; v < 7; ++v) out[v] = R(0.5) * (FL[v] + FR[v]);
     return;
   }
-  const R iden = rdiv<R, EOS>(R(1), den);
+  const R iden = rdiv(R(1), den);
   const R lpm = lp * lm;
 #pragma unroll
   for (int v = 0; v < 7; ++v) out[v] = (lp * FL[v] - lm * FR[v] + lpm * (UR[v] - UL[v])) * iden;
@@ -739,7 +749,7 @@ __device__ __forceinline__ void cell_fluid(const CellMet<R>& M, const KParams& k
   for (int i = 0; i < 3; ++i) f.ut[i] = w[1 + i];
   lower3(M.g, f.ut, f.utl);
   f.W = sqrt_w(R(1) + f.ut[0] * f.utl[0] + f.ut[1] * f.utl[1] + f.ut[2] * f.utl[2]);
-  const R iW = rdiv<R, EOS>(R(1), f.W), ia = rdiv<R, EOS>(R(1), M.alpha), isg = rdiv<R, EOS>(R(1), M.sg);
+  const R iW = rdiv(R(1), f.W), ia = rdiv(R(1), M.alpha), isg = rdiv(R(1), M.sg);
   #pragma unroll
   for (int i = 0; i < 3; ++i) {
     f.v[i] = f.ut[i] * iW;
@@ -908,22 +918,22 @@ __device__ __forceinline__ bool c2p_neg(float a) { return a < 0.f; }
 // iW = 1/W = sqrt(1 - v^2).
 template <class R>
 __device__ __forceinline__ void c2p_master(R gam, R vmax2, const C2PInv<R>& I, R mu, C2PVal<R>& E) {
-  E.x = rdiv(R(1), R(1) + mu * I.b2);
+  E.x = rdiv_n(R(1), R(1) + mu * I.b2);
   E.rbar2 = E.x * E.x * I.r2 + mu * E.x * (R(1) + E.x) * I.rb * I.rb;
   const R qbar = I.q - R(0.5) * I.b2 - R(0.5) * mu * mu * E.x * E.x * (I.b2 * I.r2 - I.rb * I.rb);
   E.v2 = mu * mu * E.rbar2;
   E.vcap = c2p_above(E.v2, vmax2);
   if (E.vcap) E.v2 = vmax2;
-  E.iW = sqrt_r(R(1) - E.v2);
+  E.iW = sqrt_n(R(1) - E.v2);   // of 0, or an ulp of 1 or more
   const R qm = qbar - mu * E.rbar2;
-  E.eps = rdiv(qm * (R(1) + E.iW) + E.v2, E.iW * (R(1) + E.iW));
+  E.eps = rdiv_n(qm * (R(1) + E.iW) + E.v2, E.iW * (R(1) + E.iW));
   E.eclamp = c2p_neg(E.eps);
   if (E.eclamp) E.eps = R(0);
   const R ge = R(1) + gam * E.eps;
   const R nuA = ge * E.iW;
-  const R nuB = rdiv(ge * (R(1) + qm), R(1) + E.eps);
+  const R nuB = rdiv_n(ge * (R(1) + qm), R(1) + E.eps);
   const R nu = rmax(nuA, nuB);
-  E.f = mu - rdiv(R(1), nu + mu * E.rbar2);
+  E.f = mu - rdiv_n(R(1), nu + mu * E.rbar2);
 }
 
 // The same f(mu) for the ideal gas with two FP64 divisions instead of four (the mixed stage's
@@ -935,13 +945,13 @@ __device__ __forceinline__ void c2p_master(R gam, R vmax2, const C2PInv<R>& I, R
 // E.en / E.ed.
 template <class R>
 __device__ __forceinline__ void c2p_master_fast(R gam, R vmax2, const C2PInv<R>& I, R mu, C2PVal<R>& E) {
-  E.x = rdiv(R(1), R(1) + mu * I.b2);
+  E.x = rdiv_n(R(1), R(1) + mu * I.b2);
   E.rbar2 = E.x * E.x * I.r2 + mu * E.x * (R(1) + E.x) * I.rb * I.rb;
   const R qbar = I.q - R(0.5) * I.b2 - R(0.5) * mu * mu * E.x * E.x * (I.b2 * I.r2 - I.rb * I.rb);
   E.v2 = mu * mu * E.rbar2;
   E.vcap = c2p_above(E.v2, vmax2);
   if (E.vcap) E.v2 = vmax2;
-  E.iW = sqrt_r(R(1) - E.v2);
+  E.iW = sqrt_n(R(1) - E.v2);   // of 0, or an ulp of 1 or more
   const R qm = qbar - mu * E.rbar2;
   const R d = E.iW * (R(1) + E.iW);
   R n = qm * (R(1) + E.iW) + E.v2;
@@ -953,7 +963,7 @@ __device__ __forceinline__ void c2p_master_fast(R gam, R vmax2, const C2PInv<R>&
   const R dn = d + n, q1 = R(1) + qm;
   const bool a_wins = rgt(E.iW * dn, q1 * d);
   const R P = a_wins ? E.iW : q1, Q = a_wins ? d : dn;
-  E.f = mu - rdiv(Q, G * P + mu * E.rbar2 * Q);
+  E.f = mu - rdiv_n(Q, G * P + mu * E.rbar2 * Q);
 }
 
 // c2p_master_fast in FP64 with what does not depend on mu formed once per cell (21 FP64 instructions for 34)
@@ -985,7 +995,7 @@ __device__ __forceinline__ void c2p_master_fast64(double gam, double vmax2, cons
 // df/dmu of the ideal gas's master function in FP32 (relative error ~1e-5), for the Newton steps on the FP64
 // f: with y = mu x, x' = -b2 x^2 and y' = x^2; the capped v^2 and the clamped eps are constants
 __device__ __forceinline__ float c2p_slope32(float gam, float vmax2, const C2PInv<float>& I, float mu) {
-  const float x = fdiv(1.f, 1.f + mu * I.b2), y = mu * x, rb2 = I.rb * I.rb, dx = -I.b2 * x * x;
+  const float x = fdiv_n(1.f, 1.f + mu * I.b2), y = mu * x, rb2 = I.rb * I.rb, dx = -I.b2 * x * x;
   const float R = x * x * I.r2 + y * (1.f + x) * rb2;
   const float dR = 2.f * x * dx * I.r2 + rb2 * (x * x * (1.f + x) + y * dx);
   const float C = I.b2 * I.r2 - rb2;
@@ -993,14 +1003,14 @@ __device__ __forceinline__ float c2p_slope32(float gam, float vmax2, const C2PIn
   const float dqm = -y * x * x * C - R - mu * dR;
   float v2 = mu * mu * R, dv2 = mu * (2.f * R + mu * dR);
   if (v2 > vmax2) { v2 = vmax2; dv2 = 0.f; }
-  const float w = sqrt_r(1.f - v2), dw = fdiv(-0.5f * dv2, w), id = fdiv(1.f, w * (1.f + w));
+  const float w = sqrt_n(1.f - v2), dw = fdiv_n(-0.5f * dv2, w), id = fdiv_n(1.f, w * (1.f + w));
   float eps = (qm * (1.f + w) + v2) * id;
   float de = (dqm * (1.f + w) + qm * dw + dv2 - eps * dw * (1.f + 2.f * w)) * id;
   if (eps < 0.f) { eps = 0.f; de = 0.f; }
-  const float ge = 1.f + gam * eps, dge = gam * de, ie = fdiv(1.f, 1.f + eps);
+  const float ge = 1.f + gam * eps, dge = gam * de, ie = fdiv_n(1.f, 1.f + eps);
   const float A = ge * w, B = ge * (1.f + qm) * ie;
   const float dn = A > B ? dge * w + ge * dw : (dge * (1.f + qm) + ge * dqm - B * de) * ie;
-  const float ig = fdiv(1.f, (A > B ? A : B) + mu * R);
+  const float ig = fdiv_n(1.f, (A > B ? A : B) + mu * R);
   return 1.f + (dn + R + mu * dR) * ig * ig;
 }
 
@@ -1011,15 +1021,15 @@ __device__ __forceinline__ float c2p_slope32(float gam, float vmax2, const C2PIn
 template <class R>
 __device__ __forceinline__ void c2p_master_tab(const TabView<R>& t, R vmax2, const C2PInv<R>& I, R mu,
                                                C2PVal<R>& E, int* khint) {
-  E.x = rdiv<R, GR_EOS_TABLE>(R(1), R(1) + mu * I.b2);
+  E.x = rdiv(R(1), R(1) + mu * I.b2);
   E.rbar2 = E.x * E.x * I.r2 + mu * E.x * (R(1) + E.x) * I.rb * I.rb;
   const R qbar = I.q - R(0.5) * I.b2 - R(0.5) * mu * mu * E.x * E.x * (I.b2 * I.r2 - I.rb * I.rb);
   E.v2 = mu * mu * E.rbar2;
   E.vcap = c2p_above(E.v2, vmax2);
   if (E.vcap) E.v2 = vmax2;
-  E.iW = sqrt_r(R(1) - E.v2);
+  E.iW = sqrt_n(R(1) - E.v2);   // of 0, or an ulp of 1 or more
   const R qm = qbar - mu * E.rbar2;
-  E.eps = rdiv<R, GR_EOS_TABLE>(qm * (R(1) + E.iW) + E.v2, E.iW * (R(1) + E.iW));
+  E.eps = rdiv(qm * (R(1) + E.iW) + E.v2, E.iW * (R(1) + E.iW));
   E.rho = I.D * E.iW;
   E.eclamp = false;
   bool cl = false;
@@ -1033,20 +1043,20 @@ __device__ __forceinline__ void c2p_master_tab(const TabView<R>& t, R vmax2, con
   *khint = k;
   if (cl) { E.eps = rexpm1(tab_T(t, t.f[1], L, k, wT)); E.eclamp = true; }
   E.p = E.rho * rexp(tab_T(t, t.f[0], L, k, wT));
-  const R h = (R(1) + E.eps) + rdiv<R, GR_EOS_TABLE>(E.p, E.rho);
+  const R h = (R(1) + E.eps) + rdiv(E.p, E.rho);
   const R nuA = h * E.iW;
-  const R nuB = rdiv<R, GR_EOS_TABLE>(h * (R(1) + qm), R(1) + E.eps);
+  const R nuB = rdiv(h * (R(1) + qm), R(1) + E.eps);
   const R nu = rmax(nuA, nuB);
-  E.f = mu - rdiv<R, GR_EOS_TABLE>(R(1), nu + mu * E.rbar2);
+  E.f = mu - rdiv(R(1), nu + mu * E.rbar2);
 }
 
 // Auxiliary function mu sqrt(h0^2 + rbar^2(mu)) - 1 whose root bounds the master root from above;
 // h0 = minimum enthalpy of the EOS (1 for the ideal gas), passed squared
 template <class R, int EOS>
 __device__ __forceinline__ R c2p_aux(const C2PInv<R>& I, R h0sq, R mu) {
-  const R x = rdiv<R, EOS>(R(1), R(1) + mu * I.b2);
+  const R x = rdiv_n<R, EOS>(R(1), R(1) + mu * I.b2);
   const R rbar2 = x * x * I.r2 + mu * x * (R(1) + x) * I.rb * I.rb;
-  return mu * sqrt_r(h0sq + rbar2) - R(1);
+  return mu * sqrt_n(h0sq + rbar2) - R(1);
 }
 
 // Illinois on [a,b] (f(a) < 0 < f(b) or reverse).  Returns 0 (root), -1 (no sign change), -2 (cap).
@@ -1061,7 +1071,7 @@ __device__ __forceinline__ int illinois(Fn f, R a, R b, R fa, R fb, R tol, int m
   if (c2p_neg(fa) == c2p_neg(fb)) return -1;
   int side = 0;
   for (int it = 1; it <= max_iter; ++it) {
-    R c = rdiv<R, EOS>(a * fb - b * fa, fb - fa);
+    R c = rdiv_n<R, EOS>(a * fb - b * fa, fb - fa);
     if (!(c2p_above(c, a) && c2p_above(b, c))) c = R(0.5) * (a + b);
     if (!(c2p_above(c, a) && c2p_above(b, c))) {
       *root = c; *hi_out = b; *iters = it;
@@ -1128,7 +1138,7 @@ __device__ __forceinline__ bool c2p_presolve32(const KParams& P, const C2PInv<do
       if (!(fa < 0.f) || !(fb >= 0.f)) return false;
       phase = 3;
     } else {
-      if (fc == 0.f) { *islope = rdiv<float, EOS>(b - a, gb - ga); a = mu; b = mu; break; }
+      if (fc == 0.f) { *islope = rdiv_n<float, EOS>(b - a, gb - ga); a = mu; b = mu; break; }
       if (fc < 0.f) {
         a = mu; fa = ga = fc;
         if (side == -1) fb *= 0.5f;
@@ -1141,18 +1151,18 @@ __device__ __forceinline__ bool c2p_presolve32(const KParams& P, const C2PInv<do
       ++k;
     }
     if (k >= 12 || !(b - a > 1e-4f * b)) break;
-    mu = rdiv<float, EOS>(a * fb - b * fa, fb - fa);
+    mu = rdiv_n<float, EOS>(a * fb - b * fa, fb - fa);
     if (!(mu > a && mu < b)) mu = 0.5f * (a + b);
     if (!(mu > a && mu < b)) break;
   }
   *lo = a;
   *hi = b;
   *khint = kh;
-  if (b > a) *islope = rdiv<float, EOS>(b - a, gb - ga);
+  if (b > a) *islope = rdiv_n<float, EOS>(b - a, gb - ga);
   float c = a - ga * *islope;
   if (!(c > a && c < b)) c = 0.5f * (a + b);
   *est = c;
-  if constexpr (EOS == GR_EOS_IDEAL) *islope = fdiv(1.f, c2p_slope32(gam, vmax2, I, c));
+  if constexpr (EOS == GR_EOS_IDEAL) *islope = fdiv_n(1.f, c2p_slope32(gam, vmax2, I, c));
   return true;
 }
 
