@@ -1256,7 +1256,7 @@ __device__ __forceinline__ int con2prim_cell(const Site& site, const KParams& P,
   const double rho_thr = P.rho_thr;
   bool atm = false, reprim = false;
   if (!finite) { st |= GR_ST_FAILED; atm = true; }
-  else if (neg64(q[0]) || gtp64(rho_thr * sg, q[0])) { st |= GR_ST_ATM_THRESHOLD; atm = true; }   // D~ < rho_thr
+  else if (gt64(rho_thr * sg, q[0])) { st |= GR_ST_ATM_THRESHOLD; atm = true; }   // D~ < rho_thr
   double isg = 0.0;
   if (!atm) {
     if constexpr (FAST) isg = M.isg;
@@ -1278,7 +1278,7 @@ __device__ __forceinline__ int con2prim_cell(const Site& site, const KParams& P,
       tab_p_eps_T<double>(P.t64, D, P.t64.x0[1], ye, &pm, &eps_min);
     }
     const double tau_min = D * eps_min + 0.5 * BB;
-    if (EOS ? tau < tau_min : neg64(tau) || gtp64(tau_min, tau)) { tau = tau_min; st |= GR_ST_TAU_FLOOR; qmod = true; }
+    if (EOS ? tau < tau_min : gt64(tau_min, tau)) { tau = tau_min; st |= GR_ST_TAU_FLOOR; qmod = true; }
     double gi[6];
     if constexpr (FAST) inv3_id(M.g, isg * isg, gi);   // 1/det = (1/sqrt(gamma))^2
     else inv3(M.g, M.det, gi);
