@@ -1369,7 +1369,7 @@ __device__ __forceinline__ int con2prim_cell(const Site& site, const KParams& P,
         mu = f2d_exact(est);
         const double thr = fmax(1e-4 * P.tol, 4.5e-16);
 #pragma unroll 1
-        for (int k = 0; k < 6; ++k) {
+        for (int k = 0; k < min(6, P.max_iter); ++k) {
           fm(mu);
           ++nevals;
           const double fc = E.f;
