@@ -278,7 +278,7 @@ template <> __device__ __forceinline__ double diff64(float a, float b) {
 // integers (exactly, but for what alignment cuts off a value many bits below the largest), and rounded once.
 // ~12 integer instructions a value and ~18 a result, against 70 cycles of a scheduler for each FP64 addition.
 // ------------------------------------------------------------------------------------------------
-// largest biased exponent of n values (2047: one is not finite)
+// largest biased exponent of N values (2047: one is not finite)
 template <int N>
 __device__ __forceinline__ uint32_t fix_exp(const double* f) {
   uint32_t e = 0;
@@ -313,12 +313,22 @@ __device__ __forceinline__ double fix_round(int64_t acc, int x) {
   const uint64_t r = (n >> 11) + ((n >> 10) & 1ull & (uint64_t)((n & 0x3ffull) != 0ull || (n & 0x800ull) != 0ull));
   return from64(sg | (((uint64_t)(uint32_t)(ex - 1) << 52) + r));
 }
-__device__ __forceinline__ double nan64() { return from64(0x7ff8000000000000ull); }
+// Sets that the fixed-point sums leave to the operators: one value is not finite, or all are so small that a result
+// could fall below the normal range (then e < 64; mostly all are zero, as a vanishing shift is)
+__device__ __forceinline__ bool fix_edge(uint32_t e) { return e - 64u >= 2047u - 64u; }
+template <int N>
+__device__ __forceinline__ bool fix_zero(const double* f) {
+  uint32_t o = 0;
+#pragma unroll
+  for (int t = 0; t < N; ++t) o |= ((uint32_t)__double2hiint(f[t]) << 1) | (uint32_t)__double2loint(f[t]);
+  return o == 0u;
+}
 
 // mean of the eight vertices of a cell (index x + 2 y + 4 z)
 __device__ __forceinline__ double mean8_64(const double f[8]) {
   const uint32_t e = fix_exp<8>(f);
-  if (e == 2047u) return nan64();
+  if (fix_edge(e))
+    return fix_zero<8>(f) ? 0.0 : mul_rare(((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])), 0.125);
   int64_t a = 0;
 #pragma unroll
   for (int t = 0; t < 8; ++t) a += fix_of<7>(f[t], e);
@@ -327,8 +337,13 @@ __device__ __forceinline__ double mean8_64(const double f[8]) {
 // the mean, and the sums of the four differences along x, y and z (each zero on a constant field)
 __device__ __forceinline__ void haar8_64(const double f[8], double* mean, double* dx, double* dy, double* dz) {
   const uint32_t e = fix_exp<8>(f);
-  if (e == 2047u) {
-    *mean = *dx = *dy = *dz = nan64();
+  if (fix_edge(e)) {
+    *mean = *dx = *dy = *dz = 0.0;
+    if (fix_zero<8>(f)) return;
+    *mean = mul_rare(((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])), 0.125);
+    *dx = ((f[1] - f[0]) + (f[3] - f[2])) + ((f[5] - f[4]) + (f[7] - f[6]));
+    *dy = ((f[2] - f[0]) + (f[3] - f[1])) + ((f[6] - f[4]) + (f[7] - f[5]));
+    *dz = ((f[4] - f[0]) + (f[5] - f[1])) + ((f[6] - f[2]) + (f[7] - f[3]));
     return;
   }
   int64_t m[8];
@@ -344,7 +359,13 @@ __device__ __forceinline__ void haar8_64(const double f[8], double* mean, double
 // the 4 x 4 Lagrange midpoint interpolant of a vertex plane, weights (-1, 9, 9, -1)/16 per axis; f[4 y + x]
 __device__ __forceinline__ double lagr16_64(const double f[16]) {
   const uint32_t e = fix_exp<16>(f);
-  if (e == 2047u) return nan64();
+  if (fix_edge(e)) {
+    if (fix_zero<16>(f)) return 0.0;
+    double s[4];
+#pragma unroll
+    for (int y = 0; y < 4; ++y) s[y] = 9.0 * (f[4 * y + 1] + f[4 * y + 2]) - (f[4 * y] + f[4 * y + 3]);
+    return mul_rare(9.0 * (s[1] + s[2]) - (s[0] + s[3]), 1.0 / 256);
+  }
   int64_t r[4];
 #pragma unroll
   for (int y = 0; y < 4; ++y) {   // 54 bits, times at most 20 per axis: 63
