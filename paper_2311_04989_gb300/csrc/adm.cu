@@ -187,12 +187,13 @@ template <> __device__ __forceinline__ float mid_weight<float, 4>(int s) {
 
 // One axis of the interpolant at a vertex from its NP cells, stride `st` apart.  FP64: the weights times 2 or 16 per
 // axis (1, 1 or -1, 9, 9, -1), so that an order-4 axis takes three FP64 instructions for four and an order-2 one one
-// for two; axis_end takes the powers of two off at the end, exactly.
+// for two, with the roundings of the sum from its low end; axis_end takes the powers of two off at the end, exactly.
+// (9 (f1 + f2) - (f0 + f3) is as long and 5 % further off: 1.42e-16 of the sources for 1.34e-16.)
 template <class R, int NP>
 __device__ __forceinline__ R axis_sum(const R* src, size_t st) {
   if constexpr (sizeof(R) == sizeof(double)) {
     if constexpr (NP == 2) return src[0] + src[st];
-    else return fma(R(9), src[st] + src[2 * st], -(src[0] + src[3 * st]));
+    else return fma(R(9), src[2 * st], fma(R(9), src[st], -src[0])) - src[3 * st];
   } else {
     R s = 0;
 #pragma unroll
