@@ -375,4 +375,34 @@ __device__ __forceinline__ double lagr16_64(const double f[16]) {
   return fix_round(9 * (r[1] + r[2]) - (r[0] + r[3]), (int)e - 1075 - 1 - 8);
 }
 
+// ------------------------------------------------------------------------------------------------
+// A one-sided FP32 bound for the atmosphere test
+// ------------------------------------------------------------------------------------------------
+// x > 0 within 2^-20 from above, from the upper half of its encoding; 0 where it is not a normal FP32 number
+__device__ __forceinline__ float above32(double x) {
+  const uint32_t h = (uint32_t)__double2hiint(x);
+  return h - 0x38200000u < 0x47a00000u - 0x38200000u ? __uint_as_float(((h - 0x38000000u) << 3) + 8u) : 0.f;
+}
+// Whether D is above thr sqrt(gamma) for certain, g: gamma_xx, gamma_yy, gamma_zz at the eight vertices of a cell.
+// thr sqrt(gamma_xx gamma_yy gamma_zz) is an upper bound for a positive definite gamma_ij (Hadamard); it is formed in FP32
+// from above with a margin of 1e-3, and given up where a product is too small to keep that margin
+__device__ __forceinline__ bool surely_above(const double g[3][8], double D, double thr) {
+  float p = 1.f;
+  bool ok = true;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    float s = 0.f;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      const float f = above32(g[c][t]);
+      ok = ok && f > 0.f;
+      s += f;
+    }
+    p *= 0.125f * s;
+    ok = ok && p > 1e-30f;
+  }
+  const float d = above32(D), t = above32(thr);   // d exceeds D by 2^-20 at most
+  return ok && t > 0.f && p < 1e30f && d > 1.001f * t * sqrtf(p);
+}
+
 }  // namespace grs

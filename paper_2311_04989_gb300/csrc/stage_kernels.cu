@@ -616,33 +616,18 @@ __global__ void __launch_bounds__(kTile) k_prim2con(const DBlock* __restrict__ b
   if (EOS) a.U[5][c] = q[0] * wv[5];
 }
 
-// x > 0 within 2^-20 from above, from the upper half of its encoding; 0 where it is not a normal FP32 number
-__device__ __forceinline__ float above32(double x) {
-  const unsigned h = (unsigned)__double2hiint(x);
-  return h - 0x38200000u < 0x47a00000u - 0x38200000u ? __uint_as_float(((h - 0x38000000u) << 3) + 8u) : 0.f;
-}
-// Whether a cell's D is above the atmosphere threshold for certain: D > thr sqrt(gamma_xx gamma_yy gamma_zz), an upper
-// bound of thr sqrt(gamma) for a positive definite gamma_ij (Hadamard), formed in FP32 from above with a margin of
-// 1e-3.  Then the FP64 metric, field and variables need not be read for the test.
+// surely_above (soft64.cuh) on the metric of a cell: then its FP64 metric, field and variables need not be read for the test
 __device__ __forceinline__ bool surely_matter(const DBlock& b, const InView<double>& m, int i, int j, int k, double D, double thr) {
   const long long v0 = b.vert + vix(b, i, j, k);
   const int sy = b.N[0] + 1, sz = sy * (b.N[1] + 1);
-  float g = 1.f;
-  bool ok = true;
+  double g[3][8];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const double* a = m.M[c == 0 ? 4 : (c == 1 ? 7 : 9)] + v0;
-    float s = 0.f;
 #pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      const float f = above32(a[(t & 1) + ((t >> 1) & 1) * sy + (t >> 2) * sz]);
-      ok = ok && f > 0.f;
-      s += f;
-    }
-    g *= 0.125f * s;
+    for (int t = 0; t < 8; ++t) g[c][t] = a[(t & 1) + ((t >> 1) & 1) * sy + (t >> 2) * sz];
   }
-  const float d = above32(D), t = above32(thr);   // d exceeds D by 2^-20 at most
-  return ok && t > 0.f && g > 0.f && g < 1e30f && d > 1.001f * t * sqrtf(g);
+  return surely_above(g, D, thr);
 }
 
 // gr_con2prim, first pass: atmosphere cells (the threshold test of con2prim on the same FP64 metric)
