@@ -170,7 +170,7 @@ __device__ __forceinline__ void face_metric(const DBlock& b, const InView<R>& m,
 #pragma unroll
     for (int c = 0; c < 10; ++c) {
       const R* a = m.M[c] + base + v00;
-            out[c] = rscale<2>((a[0] + a[s1]) + (a[s2] + a[s1 + s2]));
+      out[c] = rscale<2>((a[0] + a[s1]) + (a[s2] + a[s1 + s2]));
     }
   } else {
     const R w[4] = {R(-1.0 / 16), R(9.0 / 16), R(9.0 / 16), R(-1.0 / 16)};
@@ -1060,12 +1060,10 @@ __device__ __forceinline__ R c2p_aux(const C2PInv<R>& I, R h0sq, R mu) {
 }
 
 // Illinois on [a,b] (f(a) < 0 < f(b) or reverse).  Returns 0 (root), -1 (no sign change), -2 (cap).
-// *fresh (optional): whether the root is the point f was last evaluated at.
 template <class R, int EOS, class Fn>
 __device__ __forceinline__ int illinois(Fn f, R a, R b, R fa, R fb, R tol, int max_iter, R* root, R* hi_out,
-                                        int* iters, bool* fresh = nullptr) {
+                                        int* iters) {
   *iters = 0;
-  if (fresh) *fresh = false;
   if (rzero(fa)) { *root = a; *hi_out = a; return 0; }
   if (rzero(fb)) { *root = b; *hi_out = b; return 0; }
   if (c2p_neg(fa) == c2p_neg(fb)) return -1;
@@ -1075,12 +1073,10 @@ __device__ __forceinline__ int illinois(Fn f, R a, R b, R fa, R fb, R tol, int m
     if (!(c2p_above(c, a) && c2p_above(b, c))) c = R(0.5) * (a + b);
     if (!(c2p_above(c, a) && c2p_above(b, c))) {
       *root = c; *hi_out = b; *iters = it;
-      if (fresh) *fresh = false;   // c itself was not evaluated
       return 0;
     }
     const R fc = f(c);
     *iters = it;
-    if (fresh) *fresh = true;
     if (rzero(fc)) { *root = c; *hi_out = c; return 0; }
     if (c2p_neg(fc) == c2p_neg(fa)) {
       a = c; fa = fc;

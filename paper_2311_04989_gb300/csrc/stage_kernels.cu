@@ -133,12 +133,12 @@ __global__ void __launch_bounds__(kMaxTile) k_cellprep(const DBlock* __restrict_
   }
 }
 
-// k_cellprep_sweep<R> (order-2 metric): the same outputs, bitwise, with each vertex of the metric read
-// from memory once per tile instead of by each of its eight cells.  One CTA per SweepWork walks its tile of the
-// block along z, or a part of it on a mesh of few tiles (kSweepTarget); the vertex planes z and z + 1 of the tile (with its +1 halo in x and y) sit in shared
-// memory (cp.async, two buffers), and each thread carries the 2 x 2 plane sums of its cell column from one
-// cell to the next: the cell value is 1/8 ((f0 + f1) + (f2 + f3)) + ((f4 + f5) + (f6 + f7)) in the
-// order cell_metric sums it, the first bracket being the previous cell's second.
+// k_cellprep_sweep<R> (order-2 metric): k_cellprep with each vertex of the metric read from memory once per
+// tile instead of by each of its eight cells.  One CTA per SweepWork walks its tile of the block along z, or a
+// part of it on a mesh of few tiles (kSweepTarget); the vertex planes z and z + 1 of the tile (with its +1 halo in x
+// and y) sit in shared memory (cp.async, two buffers), and each thread carries the 2 x 2 plane sums of its cell
+// column from one cell to the next: the cell value is 1/8 ((f0 + f1) + (f2 + f3)) + ((f4 + f5) + (f6 + f7)) in the
+// order cell_metric sums it without its fixed-point form, the first bracket being the previous cell's second.
 template <class R>
 __device__ __forceinline__ void sweep_copy(R* dst, const R* src) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
@@ -395,7 +395,7 @@ __device__ __forceinline__ void update_all(const DBlock& b, const InView<R>& in,
 // Mixed path: D has no source, so D' and the atmosphere test need only the fluxes and sqrt(gamma) of
 // the FP32 metric (the same band atm_band as the FP64 test); gamma_ij and sqrt(gamma) are the values
 // cellmet_from forms, so the test is the one the full metric would give.  The other variables of a
-// matter cell are formed in k_c2p (update_all), densely packed, so that this kernel carries neither the
+// matter cell are formed in k_jobs (update_all), densely packed, so that this kernel carries neither the
 // metric derivatives nor the sources.
 template <class R, int EOS>
 __device__ __forceinline__ bool update_cell(const Work& w, const DBlock& b, const InView<R>& in,
@@ -835,9 +835,7 @@ static cudaError_t stage_fused(const DBlock* blocks, int nblocks, const KLaunch 
   cudaError_t e = launch_cellprep_sweep<float>(blocks, in, ws, st, false);
   if (e != cudaSuccess) return e;
   if (ev) cudaEventRecord(ev[2], st);
-  e = cudaMemsetAsync(ws.njobs, 0, sizeof(int), st);
-  if (e != cudaSuccess) return e;
-  e = launch_fused(blocks, nblocks, in, s, ws, kp, st);
+  e = launch_fused(blocks, nblocks, in, s, ws, kp, st);   // the cell preparation has emptied the job list
   if (e != cudaSuccess) return e;
   if (ev) {
     for (int k = 3; k <= 6; ++k) cudaEventRecord(ev[k], st);
