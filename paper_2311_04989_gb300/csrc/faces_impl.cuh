@@ -78,7 +78,7 @@ __device__ __forceinline__ void face_body(const Work& w, const DBlock& b, const 
 
 // FP32: at most 72 registers, so that 14 CTAs of 64 threads (the autotuned shape) fit on an SM: 28
 // warps instead of 24 at the ~80 the kernel would take, for 16-44 spilled bytes (measured on the two-star
-// workload: 3.60 ms at 80 registers, 3.47 ms at 72, 3.55 ms at 68); with a table, whose face physics
+// workload when set: 3.60 ms at 80 registers, 3.47 ms at 72, 3.55 ms at 68; 3.24 ms now); with a table, whose face physics
 // holds more, 80.  FP64: 128 (48 AMR-like
 // blocks: 4.60 ms; at 80 4.73, at 96 4.68, at 168 4.62).  The FP64 kernel is bound by the FP64 pipe: 7.44 ms with
 // every operation there, 6.28 ms with its divisions and roots as integers, 4.5 ms with the reconstruction in

@@ -13,7 +13,8 @@ namespace grs {
 // Launch overlap of the kernels of one stage (programmatic dependent launch): a stage kernel may be brought up while
 // its predecessor's last CTAs finish, and waits for it to be complete, memory included, before it reads or
 // writes anything.  The launch latencies of the chain then hide behind the kernels, which is what a small mesh
-// waits for (one 16^3 block: 70 -> 49 us a stage, one 64^3 star 203 -> 170, the 4096-block batch 7.08 ms either way).
+// waits for (one 16^3 block: 74 -> 59 us a stage, one 64^3 star 227 -> 213, one ragged FP64 block 190 -> 180, the 4096-block
+// batch 7.29 -> 7.27 ms, all in the default launch shapes).
 // No earlier trigger: with the successor let in as soon as all CTAs have started, its waiting CTAs took the places
 // unevenly (61 us, and one FP64 block 177 -> 230 us).  Every kernel that launch_stage_kernel may launch with
 // overlap begins with stage_begin().

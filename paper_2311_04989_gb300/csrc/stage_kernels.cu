@@ -460,7 +460,8 @@ __device__ __forceinline__ bool update_cell(const Work& w, const DBlock& b, cons
 }
 
 // FP32: at most 64 registers (four 256-thread CTAs per SM): the mixed update is bound by load latency.  FP64: 128 (48
-// AMR-like blocks: 0.72 ms at the 212 it would take, 0.62 at 128, 0.62 at 96, 0.63 at 168): FP64 pipe and latency
+// AMR-like blocks: 0.72 ms at the 212 it would take, 0.62 at 128, 0.62 at 96, 0.63 at 168; 0.69 since gamma_ij is summed in
+// FP64 as in con2prim): FP64 pipe (88 % busy) and latency
 template <class R, int EOS>
 __global__ void __maxnreg__(sizeof(R) == sizeof(float) ? 64 : 128) k_update(const DBlock* __restrict__ blocks, const Work* __restrict__ work,
                                                      int nwork, const __grid_constant__ InView<R> in,
@@ -499,8 +500,9 @@ __device__ __forceinline__ Job job_cell(const DBlock& b, int e) {
 
 // k_jobs<EOS, ORDER>: U' of the queued cells of the mixed stage (update_all on the FP32 inputs) into Uo.  A kernel of
 // its own: with con2prim in the same one, its registers and code kept the solve at 12 warps per SM and out of
-// the instruction cache (AMR-like batch, 256 blocks, 4.3 M cells: 3.40 ms together, 2.70 ms as two kernels at
-// 96 registers; at 80 2.79, at 128 2.77, at 168 3.02).  0.62 ms there, latency-bound.
+// the instruction cache (AMR-like batch, 256 blocks, 4.3 M cells: 3.40 ms together, 2.70 ms when they were parted).
+// Registers, with the k_c2p after it on that batch / on the order-4 batch of 64 x 24^3 cells: 64 2.55 / 1.08 ms, 80
+// 2.43 / 0.99, 96 2.39 / 1.00, 128 2.40 / 1.02.  0.58 ms of it, waiting on loads and on the FP64 pipe (59 %).
 template <int EOS, int ORDER>
 __global__ void __maxnreg__(96) k_jobs(const DBlock* __restrict__ blocks, const __grid_constant__ InView<float> in,
                        const __grid_constant__ StateView s, const __grid_constant__ Workspace ws,
@@ -545,12 +547,12 @@ struct PoolSite {
 // k_c2p: FP64 con2prim (Sec. 3.5, App. A) of the queued cells from the U' in Uo (left there by k_jobs, k_update,
 // the fused sweep or the caller of gr_con2prim).
 // MODE: con2prim_cell's form; every path of a mixed stage uses the same, so that they agree bitwise.
-// Bound by the FP64 pipe (75-84 % busy).  On the AMR-like batch (256 blocks, FP32 pre-solve) the FP64
-// instructions per warp went from 640 to about 230 and the time with k_jobs from 5.09 to 2.5 ms: divisions and
+// Bound by the FP64 pipe (75 % busy).  On the AMR-like batch with the FP32 pre-solve the FP64 instructions per 32 cells
+// went from about 540 to 205 (37 of them k_jobs') and the time of 256 blocks with k_jobs from 5.09 to 2.39 ms: divisions and
 // roots as integers (soft64.cuh), one evaluation site per solve, Newton steps, the cell metric by fixed-point
-// means.  Registers: NEWTON 96 (80 2.44 ms, 112 2.40, 128 2.36 with k_jobs, but a 64^3 star then 178 us for 168),
-// BRACKET and PLAIN 128 (RK3 step of 512 blocks 10.8 ms; 112 11.9, 96 12.0, 168 10.9).  gr_con2prim
-// on 64 x 32^3 cells 4.80 -> 2.47 ms (ideal gas), on 32 x 32^3 with the table 7.4 -> 4.5 ms.
+// means.  Registers: NEWTON 96 (with k_jobs 80 2.44 ms, 112 2.42, 128 2.37, but the order-4 batch 1.04 for 1.00),
+// BRACKET and PLAIN 128 (when set: RK3 step of 512 blocks 10.8 ms; 112 11.9, 96 12.0, 168 10.9).  gr_con2prim
+// on 64 x 32^3 cells 4.80 -> 2.47 ms (ideal gas), on 32 x 32^3 with the table 7.4 -> 4.4 ms.
 template <int EOS, int MODE>
 __global__ void __maxnreg__(MODE == C2P_NEWTON ? 96 : 128) k_c2p(const DBlock* __restrict__ blocks, const __grid_constant__ InView<double> in64,
                                        const __grid_constant__ StateView s, const __grid_constant__ Workspace ws,
