@@ -47,11 +47,12 @@ template <> __device__ __forceinline__ float rdiv(float a, float b) { return __f
 // __fdividef for a divisor that is not subnormal: a times the hardware reciprocal of b without the scaling of subnormal
 // divisors, the same bits otherwise, subnormal dividends and quotients included (two instructions for four to five;
 // a face takes some fifty of them: the two-star batch 7.28 ms in the default launch shapes for 7.41 without it)
-__device__ __forceinline__ float fdiv_n(float a, float b) {
+__device__ __forceinline__ float rcp_n(float b) {
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(b));
-  return __fmul_rn(a, y);
+  return y;
 }
+__device__ __forceinline__ float fdiv_n(float a, float b) { return __fmul_rn(a, rcp_n(b)); }
 // rdiv for such a divisor.  With a table it is rdiv: there another division changes which products the compiler fuses,
 // the FP32 fluxes by their rounding, and the pre-solve's bracket (and with it the status bit of a rejected one)
 template <class R, int EOS = GR_EOS_IDEAL>
@@ -943,7 +944,11 @@ __device__ __forceinline__ void c2p_master(R gam, R vmax2, const C2PInv<R>& I, R
 // with nu = G P / Q for the larger one, f = mu - 1/(nu + mu rbar^2) = mu - Q / (G P + mu rbar^2 Q).
 // The same function as c2p_master up to rounding; eps itself (needed only at the root) is left as
 // E.en / E.ed.
-template <class R>
+// FUSE (FP32): the quotient's product fused into the difference, as the compiler does with __fdividef.  f then keeps a
+// sign next to the root where the rounded product gives zero, so the pre-solve closes its bracket from both sides: the
+// bracket, and with it the rejected bit and the evaluations of gr_con2prim with GR_GUESS_FP32, hang on it.  The Newton
+// form, which only starts from the pre-solve's root, takes the zero and ends sooner (AMR-like batch 3.70 ms for 3.93).
+template <class R, bool FUSE = false>
 __device__ __forceinline__ void c2p_master_fast(R gam, R vmax2, const C2PInv<R>& I, R mu, C2PVal<R>& E) {
   E.x = rdiv_n(R(1), R(1) + mu * I.b2);
   E.rbar2 = E.x * E.x * I.r2 + mu * E.x * (R(1) + E.x) * I.rb * I.rb;
@@ -963,7 +968,9 @@ __device__ __forceinline__ void c2p_master_fast(R gam, R vmax2, const C2PInv<R>&
   const R dn = d + n, q1 = R(1) + qm;
   const bool a_wins = rgt(E.iW * dn, q1 * d);
   const R P = a_wins ? E.iW : q1, Q = a_wins ? d : dn;
-  E.f = mu - rdiv_n(Q, G * P + mu * E.rbar2 * Q);
+  const R T = G * P + mu * E.rbar2 * Q;
+  if constexpr (FUSE) E.f = __fmaf_rn(-Q, rcp_n(T), mu);
+  else E.f = mu - rdiv_n(Q, T);
 }
 
 // c2p_master_fast in FP64 with what does not depend on mu formed once per cell (21 FP64 instructions for 34)
@@ -1101,7 +1108,7 @@ __device__ __forceinline__ int illinois(Fn f, R a, R b, R fa, R fb, R tol, int m
 // *est (in (0, top]) and *islope (1/f' there): where the FP64 Newton steps of the mixed stage start; the
 // ideal gas's slope is c2p_slope32's, the table's the secant of the bracket.  *khint: the temperature
 // interval of the last evaluation (table).
-template <int EOS>
+template <int EOS, int MODE>
 __device__ __forceinline__ bool c2p_presolve32(const KParams& P, const C2PInv<double>& I64, float* lo, float* hi,
                                                float* est, float* islope, int* khint) {
   C2PInv<float> I;
@@ -1124,7 +1131,7 @@ __device__ __forceinline__ bool c2p_presolve32(const KParams& P, const C2PInv<do
   float ga = 0.f, gb = 0.f;   // f(a), f(b) as evaluated (the Illinois steps halve fa, fb)
   int phase = 0, side = 0, k = 0;
   for (;;) {
-    if constexpr (EOS == GR_EOS_IDEAL) c2p_master_fast<float>(gam, vmax2, I, mu, E);
+    if constexpr (EOS == GR_EOS_IDEAL) c2p_master_fast<float, MODE == C2P_PLAIN>(gam, vmax2, I, mu, E);
     else c2p_master_tab<float>(P.t32, vmax2, I, mu, E, &kh);
     const float fc = E.f;
     if (phase == 0) { fa = ga = fc; mu = mup; phase = 1; continue; }
@@ -1351,7 +1358,7 @@ __device__ __forceinline__ int con2prim_cell(const Site& site, const KParams& P,
     bool pre = false;      // ... and bracketed the root in [lo32, hi32]
     float lo32 = 0.f, hi32 = 0.f, est = 0.f, islope = 0.f;
     if (MODE == C2P_NEWTON || (MODE == C2P_PLAIN && P.c2p_guess == GR_GUESS_FP32)) {
-      pre = c2p_presolve32<EOS>(P, I, &lo32, &hi32, &est, &islope, &kh);
+      pre = c2p_presolve32<EOS, MODE>(P, I, &lo32, &hi32, &est, &islope, &kh);
     }
     if constexpr (MODE == C2P_NEWTON) {
       // Newton steps on the FP64 f from the FP32 estimate (error ~1e-7) with the FP32 slope (~1e-5, table
