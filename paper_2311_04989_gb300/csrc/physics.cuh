@@ -1021,6 +1021,12 @@ __device__ __forceinline__ float c2p_slope32(float gam, float vmax2, const C2PIn
   return 1.f + (dn + R + mu * dR) * ig * ig;
 }
 
+// mu rbar^2 of the table's master function: in FP64 one rounded product for both of its uses, and the secant of the solve
+// with its first product fused, so that the solve's steps do not depend on what else is evaluated with f (the compiler
+// fuses one way or the other; evaluation counts and the status at an iteration cap hang on the last bit of f)
+__device__ __forceinline__ double tmul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float tmul(float a, float b) { return a * b; }
+
 // The same master function with the tabulated EOS (Sec. 2.2.1, App. A): rho = D/W moved into the
 // table, the temperature of e/rho = 1 + eps by the exact inverse of the interpolant (eps reset to the
 // table's value at the nearest end when outside), p from the table; (1 + a)(1 + eps) = h =
@@ -1035,7 +1041,8 @@ __device__ __forceinline__ void c2p_master_tab(const TabView<R>& t, R vmax2, con
   E.vcap = c2p_above(E.v2, vmax2);
   if (E.vcap) E.v2 = vmax2;
   E.iW = sqrt_n(R(1) - E.v2);   // of 0, or an ulp of 1 or more
-  const R qm = qbar - mu * E.rbar2;
+  const R m2 = tmul(mu, E.rbar2);
+  const R qm = qbar - m2;
   E.eps = rdiv(qm * (R(1) + E.iW) + E.v2, E.iW * (R(1) + E.iW));
   E.rho = I.D * E.iW;
   E.eclamp = false;
@@ -1054,7 +1061,7 @@ __device__ __forceinline__ void c2p_master_tab(const TabView<R>& t, R vmax2, con
   const R nuA = h * E.iW;
   const R nuB = rdiv(h * (R(1) + qm), R(1) + E.eps);
   const R nu = rmax(nuA, nuB);
-  E.f = mu - rdiv(R(1), nu + mu * E.rbar2);
+  E.f = mu - rdiv(R(1), nu + m2);
 }
 
 // Auxiliary function mu sqrt(h0^2 + rbar^2(mu)) - 1 whose root bounds the master root from above;
@@ -1505,7 +1512,7 @@ __device__ __forceinline__ int con2prim_cell(const Site& site, const KParams& P,
         phase = Z;
         continue;
       }
-      double c = div64(a * fb - b * fa, fb - fa);
+      double c = div64(EOS ? fma(a, fb, -(b * fa)) : a * fb - b * fa, fb - fa);
       if (!(gtp64(c, a) && gtp64(b, c))) {
         c = 0.5 * (a + b);
         if (!(gtp64(c, a) && gtp64(b, c))) { root = c; r = 0; break; }   // c itself was not evaluated
